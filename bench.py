@@ -193,7 +193,13 @@ def roofline_for(dom: dict, peaks: dict, step_ms_total: float) -> dict:
     sm_max = peaks.get("sm_max_mhz", 2070.0)
     sms = peaks["n_sm"]
     name = dom["name"]
-    if name.startswith("conv_gemm_fp32"):
+    if name.startswith("conv_gemm_fp32_split"):
+        # FP32 products as six BF16 products each on the tensor cores
+        bound, unit = "tensor", "TFLOP/s"
+        achieved = dom["algo_flops"] / (dom["total_ms"] / 1000.0) / 1e12
+        peak = peaks.get("bf16_tflops_sustained", 1700.0) / 6.0
+        src = f"{peaks['_source']} bf16_tflops_sustained / 6 (BF16 products per FP32 product)"
+    elif name.startswith("conv_gemm_fp32"):
         bound, unit = "alu", "TFLOP/s"
         achieved = dom["algo_flops"] / (dom["total_ms"] / 1000.0) / 1e12
         peak = sms * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12

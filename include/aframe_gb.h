@@ -47,7 +47,8 @@ extern "C" {
 #define AFG_ERR_UNSUPPORTED (-8) /* configuration this build does not implement */
 
 /* precision of the network's convolutions */
-#define AFG_FP32 0 /* FP32 SIMT implicit-GEMM convolutions ("plain") */
+#define AFG_FP32 0 /* FP32 operands and accumulation ("plain"): FP32 FMAs, or, where every width is 64..512 and the
+                      context has no memory budget, exact three-term BF16 products on the tensor cores */
 #define AFG_BF16 1 /* BF16 operands, FP32 accumulation on tcgen05 tensor cores */
 
 typedef struct afg_ctx afg_ctx;

@@ -158,6 +158,7 @@ enum KernelKind {
     KK_CONVERT,
     KK_FAR,
     KK_RESAMPLE,
+    KK_CONV_SPLIT,
     KK_COUNT
 };
 extern const char *const kKernelNames[KK_COUNT];
@@ -180,12 +181,14 @@ struct Prof {
 struct BatchCache;
 struct ServeEngine;
 struct TcPlan;
+struct SplitPlan;
 
 struct afg_ctx {
     Prof prof;
     BatchCache *batch = nullptr;      // captured timeslide-batch graph (batch.cu)
     ServeEngine *serve = nullptr;     // streaming engine (serve.cu)
     TcPlan *tcplan = nullptr;         // per-layer tensor-core plan of wide networks (net_tc_layers.cu)
+    SplitPlan *splitplan = nullptr;   // FP32 network on the tensor cores (net_split.cu)
     afg_config cfg;
     int device = 0;
     std::string err;
@@ -227,6 +230,7 @@ enum {
     WS_TRIG_FLAG,
     WS_TRIG_COUNT,
     WS_FB_SCRATCH,
+    WS_RAW,
 };
 
 struct KScope {
@@ -325,10 +329,18 @@ int whiten_multi_piece_max(const afg_ctx *ctx);  // outputs per piece of launch_
 bool whiten_multi_takes_staging(const afg_ctx *ctx);  // pieces may carry stg / sc_ring
 // net_fp32.cu
 int net_plan_build(afg_ctx *ctx, const float *weights_host, int64_t n_weights);
+int infer_fp32_reserve(afg_ctx *ctx, int64_t n_win);
 int launch_infer_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first,
                       int64_t stride, int64_t n_win, int64_t shift, float *logits, cudaStream_t st);
 int launch_stem_gn_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first, int64_t stride,
                         int64_t shift, int64_t w0, int nw, float *f0, float *f1, cudaStream_t st);
+// net_split.cu
+int net_split_prepare(afg_ctx *ctx);
+void net_split_release(afg_ctx *ctx);
+bool net_split_available(const afg_ctx *ctx);
+int net_split_reserve(afg_ctx *ctx, int64_t n_win);
+int launch_infer_split(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first, int64_t stride,
+                       int64_t n_win, int64_t shift, float *logits, cudaStream_t st);
 // net_tc_layers.cu
 int net_tc_layers_prepare(afg_ctx *ctx);
 void net_tc_layers_release(afg_ctx *ctx);

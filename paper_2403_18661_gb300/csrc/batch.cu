@@ -323,10 +323,7 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
         // the FP32 network's activation workspaces at the size of the longest series
         int64_t max_win = 0;
         for (const SegDesc &d : P.segs) max_win = std::max(max_win, d.n_win);
-        int64_t per_win = ctx->plan.max_act_per_window * (int64_t)sizeof(float);
-        int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(max_win, ((int64_t)4 << 30) / per_win));
-        chunk = std::min<int64_t>(chunk, 16384);
-        for (int i = 0; i < 4 && !rc; ++i) rc = afg_ws_reserve(ctx, WS_ACT0 + i, (size_t)(chunk * per_win), &tmp);
+        rc = infer_fp32_reserve(ctx, max_win);
         if (rc) return rc;
     }
     // descriptors are uploaded synchronously: they are constant for a captured graph

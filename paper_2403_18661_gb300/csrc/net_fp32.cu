@@ -9,6 +9,9 @@
 // t*stride + (1 - pad), so every convolution is a GEMM whose A operand is a
 // strided view of the activation buffer (implicit GEMM, no im2col copy).
 //
+// Networks whose widths are all 64..512 run on the tensor cores instead
+// (net_split.cu); this path serves the others and contexts with a memory budget.
+//
 // Per conv: k_conv_fp32 (tiled SIMT GEMM) writes the raw output; then
 // k_groupnorm computes the group statistics of each window (two passes,
 // one warp per group), and applies the affine map, the optional residual and
@@ -642,16 +645,33 @@ int launch_stem_gn_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_str
 }
 
 // ---------------------------------------------------------------- forward
+// Windows per chunk of the SIMT path: each activation buffer under ~4 GiB
+static int64_t simt_chunk(const afg_ctx *ctx, int64_t n_win) {
+    const int64_t per_win = ctx->plan.max_act_per_window * (int64_t)sizeof(float);
+    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_win, ((int64_t)4 << 30) / per_win));
+    return std::min<int64_t>(chunk, 16384);
+}
+
+// Reserve what launch_infer_fp32 over n_win windows uses (a graph capture allows no allocation).
+int infer_fp32_reserve(afg_ctx *ctx, int64_t n_win) {
+    if (net_split_available(ctx)) return net_split_reserve(ctx, n_win);
+    const size_t bytes = (size_t)(simt_chunk(ctx, n_win) * ctx->plan.max_act_per_window) * sizeof(float);
+    void *tmp = nullptr;
+    int rc = AFG_OK;
+    for (int i = 0; i < 4 && !rc; ++i) rc = afg_ws_reserve(ctx, WS_ACT0 + i, bytes, &tmp);
+    return rc;
+}
+
 int launch_infer_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first, int64_t stride,
                       int64_t n_win, int64_t shift, float *logits, cudaStream_t st) {
+    if (net_split_available(ctx))
+        return launch_infer_split(ctx, y, n_y, y_stride, first, stride, n_win, shift, logits, st);
     const NetPlan &P = ctx->plan;
     const int G = P.net.groups;
     const float eps = P.net.eps;
     const int W = ctx->cfg.win_len;
-    // windows per chunk: keep each activation buffer under ~4 GiB
-    int64_t per_win = P.max_act_per_window * (int64_t)sizeof(float);
-    int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_win, ((int64_t)4 << 30) / per_win));
-    chunk = std::min<int64_t>(chunk, 16384);
+    const int64_t per_win = P.max_act_per_window * (int64_t)sizeof(float);
+    const int64_t chunk = simt_chunk(ctx, n_win);
     float *buf[4];
     for (int i = 0; i < 4; ++i) {
         int rc = afg_ws_reserve(ctx, WS_ACT0 + i, (size_t)(chunk * per_win), (void **)&buf[i]);

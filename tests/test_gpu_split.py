@@ -1,0 +1,64 @@
+"""FP32 wide networks on the tensor cores (three BF16 terms per float, net_split.cu) against the FP64 oracle,
+at the sizes where tiles, units and layouts can go wrong, and against the SIMT path a context with a memory
+budget keeps."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import oracle as orc  # noqa: E402
+from paper_2403_18661_gb300 import abi, inputs  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+LOGIT_TOL = 1e-4  # |dz| <= 1e-4 (1 + |z|): the FP32 bound of test_gpu_parity
+
+# groups 2 .. 32 give 2 to 64 channels a group; window lengths give one row to 8192 rows per window, whole and
+# ragged units of 32 positions, and tiles that hold part of a window or many
+NETS = [
+    (inputs.NetSpec(stem_k=7, stem_stride=2, stem_pool=1, widths=(64, 128, 256, 512), blocks=(1, 1, 1, 1), groups=16), 3072),
+    (inputs.NetSpec(stem_k=7, stem_stride=2, stem_pool=1, widths=(64, 128, 256, 512), blocks=(1, 2, 1, 1), groups=32), 1024),
+    (inputs.NetSpec(stem_k=3, stem_stride=1, stem_pool=0, widths=(64,), blocks=(2,), groups=32), 8192),
+    (inputs.NetSpec(stem_k=5, stem_stride=2, stem_pool=0, widths=(128, 64), blocks=(1, 1), groups=1), 160),
+    (inputs.NetSpec(stem_k=1, stem_stride=1, stem_pool=1, widths=(256, 256), blocks=(1, 1), groups=8), 96),
+    (inputs.NetSpec(stem_k=7, stem_stride=2, stem_pool=1, widths=(64, 64, 512, 64), blocks=(1, 1, 1, 1), groups=2), 64),
+]
+
+
+@pytest.mark.parametrize("case", range(len(NETS)))
+@pytest.mark.parametrize("n_win", [1, 3, 17])
+def test_split_network_matches_oracle(case, n_win):
+    net, win_len = NETS[case]
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=win_len)
+    w = inputs.make_weights(net, 11 + case)
+    stride, shift = 37, 129
+    y = np.random.default_rng(case).standard_normal((2, (n_win - 1) * stride + win_len + 200)).astype(np.float32)
+    ctx = abi.Context(wl, w)
+    yd = torch.from_numpy(y).cuda()
+    ctx.profile_enable()
+    z = ctx.infer_windows(yd, 3, stride, n_win, shift=shift).cpu().numpy()
+    assert any(k["name"] == "conv_gemm_fp32_split_tcgen05" for k in ctx.profile_read())
+    ctx.sync()
+    for j in {0, n_win // 2, n_win - 1}:
+        a = 3 + j * stride
+        l1 = np.take(y[1], np.arange(a + shift, a + shift + win_len), mode="wrap")
+        want = orc.network(net, w, np.stack([y[0, a:a + win_len], l1]).astype(np.float64))
+        assert abs(z[j] - want) <= LOGIT_TOL * (1 + abs(want)), (j, z[j], want)
+    ctx.close()
+
+
+def test_split_long_call_and_simt_path_agree():
+    """More windows than one launch sequence holds, against a budgeted context (SIMT convolutions)."""
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=inputs.RESNET34_NET)
+    w = inputs.make_weights(wl.net, 5)
+    n_win = 1027
+    y = torch.randn((2, (n_win - 1) * 16 + wl.win_len), device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    got = []
+    for budget in (0, 32 << 30):
+        ctx = abi.Context(wl, w, hbm_budget=budget)
+        got.append(ctx.infer_windows(y, 0, 16, n_win).double().cpu().numpy())
+        ctx.sync()
+        ctx.close()
+    assert np.max(np.abs(got[0] - got[1]) / (1 + np.abs(got[1]))) <= LOGIT_TOL
