@@ -41,7 +41,6 @@ from paper_2403_18661_gb300 import inputs  # noqa: E402
 
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "sm_max_mhz": 2070.0}
 FP32_LANES_PER_SM = 128
-FP64_LANES_PER_SM = 2  # GB300: 1.25 TFLOP/s FP64 nominal = 152 SMs x 2 FMA/clk x 2 x 2.07 GHz
 
 
 def n_sm() -> int:
@@ -204,11 +203,12 @@ def roofline_for(dom: dict, peaks: dict, step_ms_total: float) -> dict:
         achieved = dom["algo_flops"] / (dom["total_ms"] / 1000.0) / 1e12
         peak = sms * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
         src = f"derived: {sms} SMs (read from the device) x {FP32_LANES_PER_SM} FP32 FMA lanes x 2 x {sm_max:g} MHz"
-    elif name.startswith("filter_build_fp64"):
+    elif name.startswith("filter_build"):
+        # additions and multiplications of float pairs, 8 FP32 instructions each
         bound, unit = "alu", "TFLOP/s"
         achieved = dom["algo_flops"] / (dom["total_ms"] / 1000.0) / 1e12
-        peak = sms * FP64_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
-        src = f"derived: {sms} SMs (read from the device) x {FP64_LANES_PER_SM} FP64 FMA lanes x 2 x {sm_max:g} MHz"
+        peak = sms * FP32_LANES_PER_SM * sm_max * 1e6 / 8.0 / 1e12
+        src = f"derived: {sms} SMs (read from the device) x {FP32_LANES_PER_SM} FP32 lanes x {sm_max:g} MHz / 8"
     elif "bf16" in name:
         bound, unit = "tensor", "TFLOP/s"
         achieved = dom["algo_flops"] / (dom["total_ms"] / 1000.0) / 1e12

@@ -176,7 +176,8 @@ int afg_psd_estimate(afg_ctx *ctx, const float *x, int64_t n, int32_t n_det, int
  * output j in [0, out_len):
  *   y[d][j] = sum_{m=-F/2}^{F/2-1} g^{(e)}_m x[d][out_first + j - m],
  *   e = (epoch_len > 0) ? min(j / epoch_len, n_psd - 1) : 0,
- * with the FIR g^{(e)} built in FP64 from psd[d][e] (amplitude psd^{-1/2},
+ * with the FIR g^{(e)} built from psd[d][e] in pairs of floats (about 46 bits;
+ * in FP64 for fir_len > 2048) and its gains rounded to FP32 (amplitude psd^{-1/2},
  * zero below f_highpass, zero-phase inverse DFT on the nfft grid, periodic
  * Hann taper of length F, scale sqrt(2/fs): unit variance for white input),
  * applied in FP32 by overlap-save FFT blocks whose circular convolution

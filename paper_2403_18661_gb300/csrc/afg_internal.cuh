@@ -21,7 +21,7 @@
 constexpr int NFFT = 16384;
 constexpr int NC = NFFT / 2;
 constexpr int NBIN = NFFT / 2 + 1;
-constexpr int FILTER_LAGS = 2048;  // lags of the tapered taps the many-CTA filter build keeps
+constexpr int FILTER_LAGS = 2048;  // longest filter of the build in float pairs
 constexpr int WB = 8192;
 
 // Epochs per thread of the Welch averaging kernel; its grid's y extent is
@@ -195,9 +195,7 @@ struct afg_ctx {
     NetPlan plan;
     float *d_params = nullptr;        // all network parameters (device)
     size_t d_params_bytes = 0;
-    double2 *tw64 = nullptr;          // exp(-2 pi i k / NFFT), k < NFFT, double (filter build)
-    double *taper64 = nullptr;        // sqrt(2 / fs) taper(m) / (2 NFFT NC) at m + FILTER_LAGS / 2, m in
-                                      // [-FILTER_LAGS / 2, FILTER_LAGS / 2) (after tw64, same allocation)
+    void *filter_tab = nullptr;       // filter build's table (filter.cu): taper pairs, or FP64 twiddles
     int64_t bytes_held = 0;
     int *d_err = nullptr;             // device-side failure record (bounded waits that gave up)
     Workspace ws[32];
@@ -229,7 +227,6 @@ enum {
     WS_TRIG_B,
     WS_TRIG_FLAG,
     WS_TRIG_COUNT,
-    WS_FB_SCRATCH,
     WS_RAW,
 };
 
@@ -288,7 +285,6 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // ----------------------------------------------------------------------------
 int afg_fail(afg_ctx *ctx, int code, const char *fmt, ...);
 int afg_cuda_fail(afg_ctx *ctx, cudaError_t e, const char *what);
-size_t filter_build_scratch_bytes(const afg_ctx *ctx, int64_t nf);
 int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out);
 void batch_cache_release(afg_ctx *ctx);
 void serve_release(afg_ctx *ctx);
@@ -319,7 +315,6 @@ int launch_whiten(afg_ctx *ctx, const float *x, int64_t n, int n_det, const doub
 cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, int64_t psd_step, int64_t psd_span,
                           int hop, int fs, double *P, double *psd, cudaStream_t st);
 cudaError_t prepare_psd_kernels();
-int launch_filter(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, float *gains, cudaStream_t st);
 int launch_psd_rows(afg_ctx *ctx, const float *const *rows_dev, int n_rows, int64_t psd_span, double *psd,
                     cudaStream_t st);
 int launch_scatter_rows(afg_ctx *ctx, const float *src, float *const *dst_dev, int n_rows, int len, cudaStream_t st);
@@ -327,6 +322,9 @@ int launch_whiten_multi(afg_ctx *ctx, const WhitenPiece *pieces_dev, int n_piece
                         cudaStream_t st);
 int whiten_multi_piece_max(const afg_ctx *ctx);  // outputs per piece of launch_whiten_multi
 bool whiten_multi_takes_staging(const afg_ctx *ctx);  // pieces may carry stg / sc_ring
+// filter.cu
+int filter_prepare(afg_ctx *ctx);
+int launch_filter(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, float *gains, cudaStream_t st);
 // net_fp32.cu
 int net_plan_build(afg_ctx *ctx, const float *weights_host, int64_t n_weights);
 int infer_fp32_reserve(afg_ctx *ctx, int64_t n_win);

@@ -144,15 +144,6 @@ int afg_ctx_create(const afg_config *cfg, const float *weights_host, int64_t n_w
     afg_ctx *ctx = new afg_ctx();
     ctx->cfg = *cfg;
     cudaGetDevice(&ctx->device);
-    size_t tw_bytes = NFFT * sizeof(double2) + FILTER_LAGS * sizeof(double);
-    cudaError_t e = cudaMalloc(&ctx->tw64, tw_bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        afg_ctx_destroy(ctx);
-        return AFG_ERR_OOM;
-    }
-    ctx->bytes_held += (int64_t)tw_bytes;
-    ctx->taper64 = reinterpret_cast<double *>(ctx->tw64 + NFFT);
     if (cudaMalloc(&ctx->d_err, 256) != cudaSuccess || cudaMemset(ctx->d_err, 0, 256) != cudaSuccess) {
         cudaGetLastError();
         afg_ctx_destroy(ctx);
@@ -160,6 +151,7 @@ int afg_ctx_create(const afg_config *cfg, const float *weights_host, int64_t n_w
     }
     ctx->bytes_held += 256;
     int rc = afg_make_twiddles(ctx);
+    if (rc == AFG_OK) rc = filter_prepare(ctx);
     if (rc == AFG_OK) rc = net_plan_build(ctx, weights_host, n_weights);
     if (rc == AFG_OK) rc = net_tc_prepare(ctx);
     if (rc == AFG_OK && cfg->precision == AFG_BF16) rc = net_tc_layers_prepare(ctx);
@@ -188,7 +180,7 @@ int afg_ctx_destroy(afg_ctx *ctx) {
     if (ctx->d_err) cudaFree(ctx->d_err);
     for (float *t : ctx->rs_taps)
         if (t) cudaFree(t);
-    if (ctx->tw64) cudaFree(ctx->tw64);
+    if (ctx->filter_tab) cudaFree(ctx->filter_tab);
     delete ctx;
     return AFG_OK;
 }

@@ -1,10 +1,9 @@
-// Shared-memory FFT building blocks, templated on the complex type; the FP64
-// filter build uses them (the FP32 Welch and whitening transforms are in
-// fft16.cuh).
+// Shared-memory FFT building blocks, templated on the complex type; the one-CTA
+// FP64 build of long filters uses them (the FP32 Welch and whitening transforms are
+// in fft16.cuh).
 //
 // Complex FFT of NC = 8192 points as a Stockham auto-sort sequence of
-// radix-8 passes (8*8*8*8) plus one radix-2 pass (and of 2048 points:
-// 8*8*8*4, and of 512: 8*8*8).  Each pass reads R points
+// radix-8 passes (8*8*8*8) plus one radix-2 pass.  Each pass reads R points
 // at stride NC/R into registers, applies the twiddles, does an in-register
 // DFT of size R and writes the R results at stride Ns; in place, with a
 // barrier between the reads and the writes.  Twiddles come from a table
@@ -118,24 +117,6 @@ __device__ __forceinline__ void fft_nc(C *d, const C *tw) {
     stockham_pass<C, 8, SIGN, NT>(d, 64, tw);
     stockham_pass<C, 8, SIGN, NT>(d, 512, tw);
     stockham_pass<C, 2, SIGN, NT>(d, 4096, tw);
-}
-
-// Complex FFT of 2048 points in shared memory (radix 8, 8, 8, 4), natural order in and
-// out, unnormalised, twiddles from the same NFFT table.  Caller syncs before.
-template <typename C, int SIGN, int NT>
-__device__ __forceinline__ void fft_2048(C *d, const C *tw) {
-    stockham_pass<C, 8, SIGN, NT, 2048>(d, 1, tw);
-    stockham_pass<C, 8, SIGN, NT, 2048>(d, 8, tw);
-    stockham_pass<C, 8, SIGN, NT, 2048>(d, 64, tw);
-    stockham_pass<C, 4, SIGN, NT, 2048>(d, 512, tw);
-}
-
-// Complex FFT of 512 points in shared memory (radix 8, 8, 8), as fft_2048.
-template <typename C, int SIGN, int NT>
-__device__ __forceinline__ void fft_512(C *d, const C *tw) {
-    stockham_pass<C, 8, SIGN, NT, 512>(d, 1, tw);
-    stockham_pass<C, 8, SIGN, NT, 512>(d, 8, tw);
-    stockham_pass<C, 8, SIGN, NT, 512>(d, 64, tw);
 }
 
 // Real-FFT split after a forward complex FFT of z_j = x_{2j} + i x_{2j+1}:

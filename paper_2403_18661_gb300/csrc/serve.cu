@@ -584,14 +584,13 @@ extern "C" int afg_stream_start(afg_ctx *ctx, const afg_stream_params *p) {
     if (!rc && (cudaMalloc(&E->d_done, 16) != cudaSuccess || cudaMemset(E->d_done, 0, 16) != cudaSuccess))
         rc = AFG_ERR_CUDA;
     // the scratch of a batch of gains refreshes (up to 16 streams: the Welch periodograms of their
-    // detectors, the FP64 transforms of their filters, their PSDs and gains), reserved and counted
+    // detectors, their PSDs and gains), reserved and counted
     // against the HBM budget here, before any stream is admitted: steps never allocate, and the
     // engine thread never changes bytes_held outside E->mu
     void *tmp = nullptr;
     const int64_t K = (p->psd_len - NFFT) / hop + 1;
     E->rb_rows = 2 * std::min(p->max_streams, 16);
     if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, (size_t)E->rb_rows * K * NBIN * sizeof(double), &tmp);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_FB_SCRATCH, filter_build_scratch_bytes(ctx, E->rb_rows), &tmp);
     if (!rc && (cudaMalloc(&E->d_rf_psd, (size_t)E->rb_rows * NBIN * sizeof(double)) != cudaSuccess ||
                 cudaMalloc(&E->d_rf_gains, (size_t)E->rb_rows * NBIN * sizeof(float)) != cudaSuccess)) {
         cudaGetLastError();

@@ -1,9 +1,8 @@
-// Welch PSD, whitening-filter build and FFT-domain whitening
+// Welch PSD and FFT-domain whitening (the filter build is in filter.cu)
 // (Sec. IV, "Noise sampling" paragraph: PSD from 8 s, frequency-domain whitening,
 // 0.5 s crop at each edge; Sec. VI: PSD from the first 64 s of state).
 //
 // Kernels
-//   k_twiddles        exp(-2 pi i k / NFFT) table in double (filter build)
 //   k_periodogram     one Hann-windowed segment per CTA: FP32 real FFT in
 //                     shared memory (radix-16 passes, fft16.cuh), the window
 //                     applied to the spectrum (a three-bin convolution),
@@ -12,10 +11,6 @@
 //   k_psd_mean        FP64 mean over the K segments of each epoch (a sliding
 //                     sum over a run of epochs per thread), density scaling
 //                     and one-sided doubling
-//   k_filter_build    one (detector, epoch) per CTA, all FP64: amplitude
-//                     response psd^-1/2 above the highpass, zero-phase
-//                     inverse real FFT, Hann taper of F taps, sqrt(2/fs),
-//                     forward real FFT at the whitening size -> real gains
 //   k_whiten          one 8192-output overlap-save block per CTA: FP32 real
 //                     FFT of 8192 + F - 1 samples (zero padded to NFFT),
 //                     multiply by the epoch's gains, inverse FFT, keep the
@@ -29,35 +24,9 @@
 #include <mutex>
 
 #include "afg_internal.cuh"
-#include "fft.cuh"
 #include "fft16.cuh"
 
 namespace {
-
-constexpr int NT64 = 1024;  // threads of the FP64 filter kernel
-
-__global__ void k_twiddles(double2 *tw64) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= NFFT) return;
-    double s, c;
-    sincospi(2.0 * (double)k / (double)NFFT, &s, &c);
-    tw64[k] = make_double2(c, -s);
-}
-
-// The taper of the many-CTA filter build with its constant factors: tap[m + FILTER_LAGS / 2] =
-// sqrt(2 / fs) (1 - cos(2 pi (m + F/2) / F)) / 2 / (2 NFFT NC) for the F taps m in [-F/2, F/2), else 0.
-// The 1 / NFFT of the inverse transform, the 1 / 2 of the inverse stage's Hermitian split and the
-// 1 / NC the gains are stored with are powers of two and every later step is linear, so folding them
-// in here is exact.
-__global__ void k_taper64(double *tap, double fs, int F) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= FILTER_LAGS) return;
-    const int m = i - FILTER_LAGS / 2, half = F / 2;
-    tap[i] = (m >= -half && m < half)
-                 ? sqrt(2.0 / fs) * (0.5 - 0.5 * cospi(2.0 * (double)(m + half) / (double)F)) /
-                       (2.0 * (double)NFFT * (double)NC)
-                 : 0.0;
-}
 
 // The FP32 transforms' twiddle table (layout in fft16.cuh): entry i = exp(-i pi a_i), a_i an exact
 // binary fraction, evaluated in FP64 and rounded to FP32.
@@ -256,244 +225,6 @@ __global__ void k_psd_mean(const double *__restrict__ P, int64_t n_seg, int seg_
         const int64_t s_old = (e - 1) * seg_step, s_new = s_old + K;
         for (int q = 0; q < seg_step; ++q) acc += src[(s_new + q) * NBIN] - src[(s_old + q) * NBIN];
         dst[e * NBIN] = acc;
-    }
-}
-
-// grid (n_psd, n_det); builds the whitening gains of one (detector, epoch)
-__global__ void __launch_bounds__(NT64) k_filter_build(const double *__restrict__ psd, int64_t n_psd, double fs,
-                                                        double f_hp, int F, const double2 *__restrict__ tw,
-                                                        float *__restrict__ gains) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2 *d = reinterpret_cast<double2 *>(smem_raw);
-    const int64_t e = blockIdx.x;
-    const int det = blockIdx.y;
-    const double *p = psd + ((int64_t)det * n_psd + e) * NBIN;
-    // amplitude response: psd^-1/2 at and above the highpass, zero below
-    for (int k = threadIdx.x; k < NBIN; k += NT64) {
-        double f = (double)k * fs / (double)NFFT;
-        double pk = p[k];
-        double a = (f >= f_hp && pk > 0.0) ? rsqrt(pk) : 0.0;
-        d[k] = make_double2(a, 0.0);
-    }
-    __syncthreads();
-    // zero-phase impulse response h = IDFT_NFFT(A) / NFFT (real, even)
-    real_split_inverse<double2, NT64>(d, tw);
-    fft_nc<double2, +1, NT64>(d, tw);
-    // taper to F taps about m = 0 and rescale; zero every other sample.
-    // Sample i of the circular buffer is lag m = i (i < NFFT/2) or i - NFFT.
-    const double norm = sqrt(2.0 / fs) / (double)NC;
-    double *t = reinterpret_cast<double *>(d);
-    const int half = F / 2;
-    for (int i = threadIdx.x; i < NFFT; i += NT64) {
-        int m = i < NFFT / 2 ? i : i - NFFT;
-        double v = 0.0;
-        if (m >= -half && m < half) {
-            double taper = 0.5 - 0.5 * cospi(2.0 * (double)(m + half) / (double)F);
-            v = t[i] * norm * taper;
-        }
-        t[i] = v;
-    }
-    __syncthreads();
-    // gains G_k = DFT_NFFT(g)_k (real for the even g); stored divided by NC,
-    // the factor the inverse half-length transform of k_whiten leaves over
-    fft_nc<double2, -1, NT64>(d, tw);
-    real_split_forward<double2, NT64>(d, tw);
-    float *out = gains + ((int64_t)det * n_psd + e) * NBIN;
-    for (int k = threadIdx.x; k < NBIN; k += NT64) out[k] = (float)(d[k].x / (double)NC);
-}
-
-// ---- filter build spread over many CTAs (fir_len <= 2048).  With the 16384-point grid
-// N, P sub-transforms of L = N / P points (L = 2048, or 512 when few filters are built):
-//   inverse:  h_m = (1/N) sum_r e^{+2 pi i r m / N} Z_r[m mod L],
-//             Z_r = sum_j A_{P j + r} e^{+2 pi i j n / L}      (P inverse FFTs of L points)
-//   taper:    g_m = sqrt(2/fs) taper(m) h_m,  m in [-1024, 1024) (the F <= 2048 taps lie inside)
-//   forward:  G_{P j + r} = sum_n y_r[n] e^{-2 pi i j n / L},
-//             y_r[n] = sum_{m = n mod L} g_m e^{-2 pi i r m / N}   (P forward FFTs of L points;
-//             at L = 2048 each slot n holds one lag, at L = 512 it folds four)
-// The same FP64 arithmetic as k_filter_build (up to rounding order), on many CTAs per filter
-// instead of one.  A and G are real and even in k, so residue P - r is residue r reversed:
-// A_{P j + P - r} = A_{P (L - 1 - j) + r}, hence Z_{P-r}[n] = e^{-2 pi i n / L} conj Z_r[n], and
-// the same for G.  Only the residues r = 0 .. P/2 are transformed:
-//   h_m = (1/N) (Re Z_0[n] + Re(e^{+2 pi i (P/2) m / N} Z_{P/2}[n]) + 2 sum_{0<r<P/2} Re(e^{+2 pi i r m / N} Z_r[n]))
-// and G at bins k > N/2 of residues 0 < r < P/2 is written to bin N - k (residue P - r).
-// Each stage pairs two real sub-transforms into one complex FFT (real amplitude response;
-// Hermitian folded taps): CTA (b, f) takes residues (0, P/2) of filter f for b = 0, (2b - 1, 2b)
-// for 0 < b < P/4, and for b = P/4 residue P/2 - 1 of the filters f and f + 1 (f even; the
-// CTAs of odd f at b = P/4 have no work).  P / 4 + 1 CTAs per filter and stage.
-constexpr int FB_LAGS = FILTER_LAGS;  // lags m in [-FB_LAGS / 2, FB_LAGS / 2)
-constexpr int FB_T = 256;
-
-template <int L>
-__device__ __forceinline__ void fb_fft(double2 *d, const double2 *tw, bool inverse) {
-    if (L == 2048) {
-        if (inverse) fft_2048<double2, +1, FB_T>(d, tw);
-        else fft_2048<double2, -1, FB_T>(d, tw);
-    } else {
-        if (inverse) fft_512<double2, +1, FB_T>(d, tw);
-        else fft_512<double2, -1, FB_T>(d, tw);
-    }
-}
-
-// The two real sub-transforms (filter f1, residue r1) and (f2, r2) of CTA (b, f) of the inverse
-// and forward stages (r2 < 0: the first alone); false for a CTA without work.
-template <int P>
-__device__ __forceinline__ bool fb_task(int b, int64_t f, int64_t nf, int64_t &f1, int &r1, int64_t &f2, int &r2) {
-    f1 = f2 = f;
-    if (b < P / 4) {
-        r1 = b == 0 ? 0 : 2 * b - 1;
-        r2 = b == 0 ? P / 2 : 2 * b;
-        return true;
-    }
-    if (f & 1) return false;
-    r1 = r2 = P / 2 - 1;
-    f2 = f + 1;
-    if (f2 >= nf) r2 = -1;
-    return true;
-}
-
-// grid (P / 4 + 1, n_filters): Z_r1 of filter f1 and Z_r2 of filter f2 (fb_task; filter
-// f = det * n_psd + e) from one complex transform.  Both inputs A_{P j + r} are real, so each Z
-// is Hermitian and C = IFFT(A_r1 + i A_r2) splits as 2 Z_r1[n] = C[n] + conj C[-n],
-// 2 Z_r2[n] = (C[n] - conj C[-n]) / i.  Z holds 2 Z_r (the 1/2 is in the taper table).
-template <int L>
-__global__ void __launch_bounds__(FB_T) k_fb_inverse(const double *__restrict__ psd, double fs, double f_hp,
-                                                     const double2 *__restrict__ tw, double2 *__restrict__ Z) {
-    constexpr int P = NFFT / L;
-    __shared__ double2 d[L];
-    int r1, r2;
-    int64_t f1, f2;
-    if (!fb_task<P>(blockIdx.x, blockIdx.y, gridDim.y, f1, r1, f2, r2)) return;
-    // The highpass test fr >= f_hp with fr = kk fs / NFFT, as the first bin k_hp that passes it (the same
-    // FP64 expression, evaluated once per thread), and pk > 0 as a test of its bits (a positive finite or
-    // infinite double; NaN and -0 fail as they do in the FP64 comparison): no FP64 instruction per bin but
-    // the reciprocal square root.
-    const double k0 = floor(f_hp * (double)NFFT / fs) - 1.0;
-    int k_hp = f_hp != f_hp ? NFFT / 2 + 1 : k0 <= 0.0 ? 0 : k0 >= (double)NFFT ? NFFT / 2 + 1 : (int)k0;  // NaN: none
-    while (k_hp <= NFFT / 2 && (double)k_hp * fs / (double)NFFT < f_hp) ++k_hp;
-    auto amp = [&](const double *p, int k) {
-        const int kk = k <= NFFT / 2 ? k : NFFT - k;  // the amplitude response is even in k
-        const double pk = p[kk];
-        const long long b = __double_as_longlong(pk);
-        return (kk >= k_hp && b > 0 && b <= 0x7FF0000000000000LL) ? rsqrt(pk) : 0.0;
-    };
-    const double *p1 = psd + f1 * NBIN, *p2 = psd + f2 * NBIN;
-    if (blockIdx.x == 0) {
-        // residues 0 and P/2 are their own mirrors: A_{P j} = A_{P (L - j)}, A_{P j + P/2} = A_{P (L - 1 - j) + P/2};
-        // each amplitude is evaluated once and copied to its mirror
-        for (int j = threadIdx.x; j <= L / 2; j += FB_T) {
-            d[j].x = amp(p1, P * j);
-            if (j < L / 2) d[j].y = amp(p1, P * j + P / 2);
-        }
-        __syncthreads();
-        for (int j = L / 2 + threadIdx.x; j < L; j += FB_T) {
-            if (j > L / 2) d[j].x = d[L - j].x;
-            d[j].y = d[L - 1 - j].y;
-        }
-    } else {
-        for (int j = threadIdx.x; j < L; j += FB_T)
-            d[j] = make_double2(amp(p1, P * j + r1), r2 >= 0 ? amp(p2, P * j + r2) : 0.0);
-    }
-    __syncthreads();
-    fb_fft<L>(d, tw, true);
-    double2 *z1 = Z + (f1 * P + r1) * L, *z2 = Z + (f2 * P + (r2 >= 0 ? r2 : 0)) * L;
-    for (int n = threadIdx.x; n < L; n += FB_T) {
-        const double2 c = d[n], cm = d[(L - n) & (L - 1)];
-        z1[n] = make_double2(c.x + cm.x, c.y - cm.y);        // 2 Z_r1 (the 1/2 is in the taper table)
-        if (r2 >= 0) z2[n] = make_double2(c.y + cm.y, cm.x - c.x);  // 2 Z_r2
-    }
-}
-
-// g_m of lag m from the P partial transforms (slot m mod L), with the taper table tap
-template <int P, int L>
-__device__ __forceinline__ double fb_tap(const double2 *__restrict__ Zf, int m, const double *__restrict__ tap,
-                                         const double2 *__restrict__ tw) {
-    const int slot = m & (L - 1);
-    double s = 0.0;
-#pragma unroll 8
-    for (int r = 1; r < P / 2; ++r) {
-        const double2 w = tw[(r * m) & (NFFT - 1)];  // e^{-2 pi i r m / N}; use its conjugate
-        const double2 v = Zf[(int64_t)r * L + slot];
-        s += w.x * v.x + w.y * v.y;  // Re(conj(w) v)
-    }
-    const double2 wh = tw[((P / 2) * m) & (NFFT - 1)], vh = Zf[(int64_t)(P / 2) * L + slot];
-    const double h = Zf[slot].x + (wh.x * vh.x + wh.y * vh.y) + 2.0 * s;
-    return h * tap[m + FB_LAGS / 2];
-}
-
-// L = 2048: grid (FB_LAGS / FB_T, n_filters), one lag per thread, one lag per slot
-__global__ void __launch_bounds__(FB_T) k_fb_taper(const double2 *__restrict__ Z, const double *__restrict__ tap,
-                                                   const double2 *__restrict__ tw, double2 *__restrict__ Y) {
-    constexpr int L = 2048, P = NFFT / L;
-    const int64_t f = blockIdx.y;
-    const int m = blockIdx.x * FB_T + threadIdx.x - FB_LAGS / 2;  // lag in [-1024, 1024)
-    const double g = fb_tap<P, L>(Z + f * P * L, m, tap, tw);
-    double2 *y = Y + f * P * L + (m & (L - 1));
-#pragma unroll
-    y[0] = make_double2(g, 0.0);  // residue 0: twiddle 1
-#pragma unroll
-    for (int r = 1; r <= P / 2; ++r) {  // the other residues the forward stage transforms
-        const double2 w = tw[(r * m) & (NFFT - 1)];
-        y[(int64_t)r * L] = make_double2(g * w.x, g * w.y);
-    }
-}
-
-// L = 512: grid (L / FB_FS, n_filters), FB_FS slots x 4 lags per CTA.  Thread (slot n, lag t)
-// forms g_m of m = n + L t - 1024, then y_r[n] for every fourth r <= P/2 from r = t, summed over
-// the slot's four lags.
-constexpr int FB_FS = 32;
-__global__ void __launch_bounds__(FB_FS * 4) k_fb_taper_fold(const double2 *__restrict__ Z,
-                                                             const double *__restrict__ tap,
-                                                             const double2 *__restrict__ tw,
-                                                             double2 *__restrict__ Y) {
-    constexpr int L = 512, P = NFFT / L, FOLD = FB_LAGS / L;
-    static_assert(FOLD == 4, "four lags per slot");
-    __shared__ double gs[FOLD][FB_FS];
-    const int64_t f = blockIdx.y;
-    const int nl = threadIdx.x % FB_FS, t = threadIdx.x / FB_FS;
-    const int n = blockIdx.x * FB_FS + nl;
-    gs[t][nl] = fb_tap<P, L>(Z + f * P * L, n + L * t - FB_LAGS / 2, tap, tw);
-    __syncthreads();
-    double2 *y = Y + f * P * L + n;
-    for (int r = t; r <= P / 2; r += FOLD) {  // the residues the forward stage transforms
-        double ax = 0.0, ay = 0.0;
-#pragma unroll
-        for (int u = 0; u < FOLD; ++u) {
-            const int m = n + L * u - FB_LAGS / 2;
-            const double2 w = tw[(r * m) & (NFFT - 1)];
-            ax += gs[u][nl] * w.x;
-            ay += gs[u][nl] * w.y;
-        }
-        y[(int64_t)r * L] = make_double2(ax, ay);
-    }
-}
-
-// grid (P / 4 + 1, n_filters): gains G_k / NC for k <= NFFT / 2 of the residue r1 of filter f1
-// and r2 of f2 (fb_task) from one complex transform.  The taps are even, so each y_r is Hermitian and its transform
-// real: FFT(y_r1 + i y_r2) = G_{P j + r1} + i G_{P j + r2}.  Bins k > NFFT / 2 of residues
-// 0 < r < P/2 give bin NFFT - k (G is even), which belongs to residue P - r.
-template <int L>
-__global__ void __launch_bounds__(FB_T) k_fb_forward(const double2 *__restrict__ Y, const double2 *__restrict__ tw,
-                                                     float *__restrict__ gains) {
-    constexpr int P = NFFT / L;
-    __shared__ double2 d[L];
-    int r1, r2;
-    int64_t f1, f2;
-    if (!fb_task<P>(blockIdx.x, blockIdx.y, gridDim.y, f1, r1, f2, r2)) return;
-    const double2 *y1 = Y + (f1 * P + r1) * L, *y2 = Y + (f2 * P + (r2 >= 0 ? r2 : 0)) * L;
-    for (int n = threadIdx.x; n < L; n += FB_T) {
-        const double2 a = y1[n], b = r2 >= 0 ? y2[n] : make_double2(0.0, 0.0);
-        d[n] = make_double2(a.x - b.y, a.y + b.x);
-    }
-    __syncthreads();
-    fb_fft<L>(d, tw, false);
-    auto put = [&](float *out, int r, int k, double v) {
-        if (k <= NFFT / 2) out[k] = (float)v;  // G_k / NC (the 1 / NC is in the taper table)
-        else if (r != 0 && r != P / 2) out[NFFT - k] = (float)v;
-    };
-    float *out1 = gains + f1 * NBIN, *out2 = gains + f2 * NBIN;
-    for (int j = threadIdx.x; j < L; j += FB_T) {
-        put(out1, r1, P * j + r1, d[j].x);
-        if (r2 >= 0) put(out2, r2, P * j + r2, d[j].y);
     }
 }
 
@@ -857,58 +588,11 @@ int set_attrs(afg_ctx *ctx) {
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi_s, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM_S));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_filter_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)((NC + 1) * sizeof(double2))));
     g_attrs_set = true;
     return AFG_OK;
 }
 
 }  // namespace
-
-// device scratch of building nf filters at once: two FP64 complex transforms of NFFT points per
-// filter for the many-CTA build (fir_len <= 2048), none for the one-CTA build
-size_t filter_build_scratch_bytes(const afg_ctx *ctx, int64_t nf) {
-    if (ctx->cfg.fir_len > FB_LAGS || nf > 65535) return 0;
-    return (size_t)2 * nf * NFFT * sizeof(double2);
-}
-
-// gains [n_det][n_psd][NBIN] from psd: the many-CTA FP64 build where fir_len <= 2048,
-// else one CTA per filter
-int filter_build(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, float *gains, cudaStream_t st) {
-    const int64_t nf = (int64_t)n_det * n_psd;
-    if (nf <= 0) return AFG_OK;
-    // algorithmic FP64 work of one filter: an inverse and a forward transform of a real, even
-    // sequence of NFFT points (the amplitude response and the taps), 1.25 N log2 N flops each
-    // (half of a real FFT's 2.5 N log2 N)
-    const double flops = (double)nf * 2.0 * 1.25 * NFFT * 14.0;
-    static_assert(NFFT == 1 << 14, "flop count assumes log2(NFFT) = 14");
-    if (ctx->cfg.fir_len <= FB_LAGS && nf <= 65535) {
-        void *scr = nullptr;
-        int rc = afg_ws_reserve(ctx, WS_FB_SCRATCH, filter_build_scratch_bytes(ctx, nf), &scr);
-        if (rc) return rc;
-        double2 *Z = static_cast<double2 *>(scr), *Y = Z + nf * NFFT;
-        KScope ks(ctx, st, KK_FILTER, flops, (double)nf * NBIN * (8.0 + 4.0));
-        if (nf * (NFFT / 2048) >= 152) {  // enough filters to fill the GPU with 2048-point transforms
-            constexpr int L = 2048, P = NFFT / L;
-            k_fb_inverse<L><<<dim3(P / 4 + 1, (unsigned)nf), FB_T, 0, st>>>(psd, (double)ctx->cfg.fs,
-                                                                        ctx->cfg.f_highpass, ctx->tw64, Z);
-            k_fb_taper<<<dim3(FB_LAGS / FB_T, (unsigned)nf), FB_T, 0, st>>>(Z, ctx->taper64, ctx->tw64, Y);
-            k_fb_forward<L><<<dim3(P / 4 + 1, (unsigned)nf), FB_T, 0, st>>>(Y, ctx->tw64, gains);
-        } else {  // few filters: 32 sub-transforms of 512 points each (16 paired transforms per stage)
-            constexpr int L = 512, P = NFFT / L;
-            k_fb_inverse<L><<<dim3(P / 4 + 1, (unsigned)nf), FB_T, 0, st>>>(psd, (double)ctx->cfg.fs,
-                                                                        ctx->cfg.f_highpass, ctx->tw64, Z);
-            k_fb_taper_fold<<<dim3(L / FB_FS, (unsigned)nf), FB_FS * 4, 0, st>>>(Z, ctx->taper64, ctx->tw64, Y);
-            k_fb_forward<L><<<dim3(P / 4 + 1, (unsigned)nf), FB_T, 0, st>>>(Y, ctx->tw64, gains);
-        }
-    } else {
-        KScope ks(ctx, st, KK_FILTER, flops, (double)nf * NBIN * (8.0 + 4.0));
-        k_filter_build<<<dim3((unsigned)n_psd, n_det), NT64, (NC + 1) * sizeof(double2), st>>>(
-            psd, n_psd, (double)ctx->cfg.fs, ctx->cfg.f_highpass, ctx->cfg.fir_len, ctx->tw64, gains);
-    }
-    AFG_LAUNCH_CHECK(ctx, "filter build");
-    return AFG_OK;
-}
 
 // Fill the FP32 twiddle table of the current device once per process (it is a per-module device variable;
 // every context on the device and the context-free Welch entry point share it).  Synchronous: the table is
@@ -934,13 +618,6 @@ static cudaError_t ensure_tw32() {
 }
 
 int afg_make_twiddles(afg_ctx *ctx) {
-    {
-        KScope ks(ctx, 0, KK_TWIDDLES, 0.0, (double)NFFT * sizeof(double2));
-        k_twiddles<<<NFFT / 256, 256>>>(ctx->tw64);
-        if (ctx->cfg.fir_len <= FILTER_LAGS)
-            k_taper64<<<FILTER_LAGS / 256, 256>>>(ctx->taper64, (double)ctx->cfg.fs, ctx->cfg.fir_len);
-    }
-    AFG_LAUNCH_CHECK(ctx, "k_twiddles");
     if (ensure_tw32() != cudaSuccess) return AFG_ERR_CUDA;
     return set_attrs(ctx);
 }
@@ -979,7 +656,7 @@ int launch_whiten(afg_ctx *ctx, const float *x, int64_t n, int n_det, const doub
     float *gains = nullptr;
     int rc = afg_ws_reserve(ctx, WS_FILTER, (size_t)n_det * n_psd * NBIN * sizeof(float), (void **)&gains);
     if (rc) return rc;
-    rc = filter_build(ctx, psd, n_det, n_psd, gains, st);
+    rc = launch_filter(ctx, psd, n_det, n_psd, gains, st);
     if (rc) return rc;
     if (out_len <= 0) return AFG_OK;
     const WhitenLayout wl = whiten_layout(out_len, epoch_len, ctx->cfg.fir_len);
@@ -1011,11 +688,6 @@ bool whiten_multi_takes_staging(const afg_ctx *ctx) { return whiten_piece_max_s(
 int whiten_multi_piece_max(const afg_ctx *ctx) {
     const int m = whiten_piece_max_s(ctx->cfg.fir_len);
     return m ? m : WB;
-}
-
-// Filter build only: gains [n_det][n_psd][NBIN] from psd (FP64), on st.
-int launch_filter(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, float *gains, cudaStream_t st) {
-    return filter_build(ctx, psd, n_det, n_psd, gains, st);
 }
 
 // One PSD per row of psd_span samples, row r starting at rows_dev[r] (device array of n_rows
