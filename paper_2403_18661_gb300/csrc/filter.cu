@@ -10,7 +10,7 @@
 // gains are FP32, so the pairs' error is 2^-20 of their rounding.  This GPU retires 2 FP64 FMAs a clock and SM
 // against 128 FP32 ones, and a pair operation takes 8 FP32 instructions: three FP64 kernels with their
 // intermediate transforms in memory took 5.0 ms for 5402 filters (FP64 pipe 85 % busy) and 41 us for two; this
-// takes 0.97 ms and 41 us, and the whitened strain differs by 7e-10 of its norm (its error is 1.2e-6).
+// takes 0.95 ms and 30 us, and the whitened strain differs by 7e-10 of its norm (its error is 1.2e-6).
 // k_filter_build (longer filters): one CTA per filter, FP64.
 #include <math.h>
 
@@ -298,8 +298,7 @@ __device__ __forceinline__ dd amplitude(long long b, int s) {
 // filters (f: the real and the imaginary part of C conj(w_3)).
 //
 // One CTA builds NF filters with 2 NF + 1 transforms side by side, 128 threads each; amplitudes, taps and gains
-// stay in shared memory, so a filter costs one read of its PSD (a second from L2 for the scale) and one write of
-// its gains.  Amplitudes are scaled by the power of two that brings the largest near 1 (strain PSDs are near
+// stay in shared memory, so a filter costs one read of its PSD and one write of its gains.  Amplitudes are scaled by the power of two that brings the largest near 1 (strain PSDs are near
 // 1e-46), undone in the gains.  NF = 2 shares residue 3 (5 transforms for two filters instead of 6).
 // Bound by the FP32 pipe.
 template <int NF>
@@ -327,31 +326,40 @@ __global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__
     const int n_here = (int)min((int64_t)NF, nf - f0);
     float4 *d = reinterpret_cast<float4 *>(smem_raw) + g * FSLOTS;
 
-    // ---- amplitudes
+    // ---- amplitudes: every PSD value is loaded once, all loads in flight together
+    constexpr int PER = (NF * NBIN + Geo::T - 1) / Geo::T;
     if (tid < NF) emin[tid] = 1 << 20;
-    __syncthreads();
-    auto bits = [&](int f, int k) {
-        const long long b = __ldg(reinterpret_cast<const long long *>(psd) + (f0 + f) * NBIN + k);
-        return k >= k_hp && b > 0 && b < 0x7FF0000000000000LL ? b : 0LL;  // (infinity: amplitude 0)
-    };
-    for (int f = 0; f < n_here; ++f) {
-        int e = 1 << 20;
-        for (int k = tid; k < NBIN; k += Geo::T) {
-            const long long b = bits(f, k);
-            if (b) e = min(e, exp_of(b));
-        }
-        e = __reduce_min_sync(0xffffffffu, e);
-        if ((tid & 31) == 0) atomicMin(&emin[f], e);
+    long long b[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int x = tid + i * Geo::T, k = NF == 1 || x < NBIN ? x : x - NBIN;
+        b[i] = x < n_here * NBIN ? __ldg(reinterpret_cast<const long long *>(psd) + f0 * NBIN + x) : 0LL;
+        if (k < k_hp || b[i] >= 0x7FF0000000000000LL) b[i] = 0LL;  // (infinity: amplitude 0; NaN; negative stays < 0)
     }
     __syncthreads();
-    for (int f = 0; f < NF; ++f) {
-        const int s = emin[f] < (1 << 20) ? (emin[f] - 1023) >> 1 : 0;
-        for (int k = tid; k < NBIN; k += Geo::T) {
-            const long long b = f < n_here ? bits(f, k) : 0LL;
-            dd a = {0.f, 0.f};
-            if (b) a = amplitude(b, s);
-            amp[(f * FP + (k & 7)) * Geo::ARS + (k >> 3)] = make_float2(a.h, a.l);
+    int e[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) e[f] = 1 << 20;
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (b[i] > 0) {
+            const int x = exp_of(b[i]), f = NF == 1 || tid + i * Geo::T < NBIN ? 0 : NF - 1;
+            if (f == 0) e[0] = min(e[0], x);
+            else e[NF - 1] = min(e[NF - 1], x);
         }
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        e[f] = __reduce_min_sync(0xffffffffu, e[f]);
+        if ((tid & 31) == 0) atomicMin(&emin[f], e[f]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int x = tid + i * Geo::T, f = NF == 1 || x < NBIN ? 0 : NF - 1, k = x - f * NBIN;
+        if (x >= NF * NBIN) break;
+        dd a = {0.f, 0.f};
+        if (b[i] > 0) a = amplitude(b[i], (emin[f] - 1023) >> 1);
+        amp[(f * FP + (k & 7)) * Geo::ARS + (k >> 3)] = make_float2(a.h, a.l);
     }
     __syncthreads();
 
