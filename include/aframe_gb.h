@@ -160,7 +160,8 @@ int afg_wait_check(afg_ctx *ctx, int64_t limit_ns, int32_t n_blocks, int64_t *wa
  * samples every hop samples, each multiplied by the periodic Hann window,
  * transformed with a real FFT in FP32, squared in FP32 after an exact
  * power-of-two scaling of the segment's spectrum (so that no square under- or
- * overflows; relative rounding 1.2e-7) and summed in FP64:
+ * overflows; relative rounding 1.2e-7) and summed in pairs of floats (about 46
+ * bits; in FP64 for more than 16 segments or segments 2^40 apart):
  *   psd[d][e][k] = c_k / (K fs sum w^2) sum_s |X_s(k)|^2, k in [0, nfft/2],
  *   c_k = 1 for k = 0 and k = nfft/2, else 2.
  * x: [n_det][n] float32.  psd: [n_det][n_psd][nfft/2+1] float64.
@@ -547,12 +548,12 @@ int afg_fused_tuning_set(afg_ctx *ctx, const afg_fused_tuning *in);
  * allocates its workspaces on first use, so such callers use this instead.
  *
  * Result: exactly what afg_psd_estimate computes (same kernels, same
- * arguments, nfft = 16384, periodic Hann, FP32 FFT, FP64 averaging), but
+ * arguments, nfft = 16384, periodic Hann, FP32 FFT, the same sums), but
  * without a context: fs and hop are passed directly.
  * x: [n_det][n] float32 (device); psd: [n_det][n_psd][8193] float64 (device).
  *
  * Memory: the periodogram scratch (AFG_NOALLOC_MAX_PERIODOGRAMS x 8193
- * doubles, 4.2 MB) and the FP32 transforms' twiddle table (60 KB) are static
+ * floats and an exponent, 2.1 MB) and the FP32 transforms' twiddle table (60 KB) are static
  * __device__ arrays that every GPU which loads the library holds until the
  * process exits.
  * This call allocates and frees nothing.  It refuses with AFG_ERR_BUDGET

@@ -24,6 +24,9 @@ constexpr int NBIN = NFFT / 2 + 1;
 constexpr int FILTER_LAGS = 2048;  // longest filter of the build in float pairs
 constexpr int WB = 8192;
 
+// Bytes of the periodograms of n segments: FP32 rows of NBIN values and the segment's exponent.
+inline size_t periodogram_bytes(int64_t n) { return (size_t)n * (NBIN + 3) * sizeof(float); }
+
 // Epochs per thread of the Welch averaging kernel; its grid's y extent is
 // ceil(n_psd / PSD_EPT), which must stay within 65535.
 constexpr int PSD_EPT = 32;
@@ -313,7 +316,7 @@ int launch_whiten(afg_ctx *ctx, const float *x, int64_t n, int n_det, const doub
                   int64_t out_first, int64_t out_len, int64_t epoch_len, float *y, int64_t y_stride,
                   cudaStream_t st, int64_t x_stride = 0);
 cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, int64_t psd_step, int64_t psd_span,
-                          int hop, int fs, double *P, double *psd, cudaStream_t st);
+                          int hop, int fs, float *P, double *psd, cudaStream_t st);
 cudaError_t prepare_psd_kernels();
 int launch_psd_rows(afg_ctx *ctx, const float *const *rows_dev, int n_rows, int64_t psd_span, double *psd,
                     cudaStream_t st);

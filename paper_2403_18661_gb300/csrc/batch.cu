@@ -310,7 +310,7 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
     SeriesDesc *series_dev = nullptr;
     rc = afg_ws_reserve(ctx, WS_PSD, (size_t)2 * P.max_ep * NBIN * sizeof(double), (void **)&psd);
     if (!rc) rc = afg_ws_reserve(ctx, WS_WHITE, (size_t)2 * P.total_white * sizeof(float), (void **)&white);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, (size_t)2 * P.max_nseg * NBIN * sizeof(double), &tmp);
+    if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, periodogram_bytes(2 * P.max_nseg), &tmp);
     if (!rc) rc = afg_ws_reserve(ctx, WS_FILTER, (size_t)2 * P.max_ep * NBIN * sizeof(float), &tmp);
     if (!rc && !lg) rc = afg_ws_reserve(ctx, WS_LOGITS, (size_t)P.total_win * sizeof(float), (void **)&lg);
     if (!rc) rc = afg_ws_reserve(ctx, WS_BATCH_SEGS, P.segs.size() * sizeof(SegDesc), (void **)&segs_dev);

@@ -18,12 +18,12 @@ namespace {
 constexpr int kMaxPeriodograms = AFG_NOALLOC_MAX_PERIODOGRAMS;
 constexpr int kMaxDevices = 64;
 
-// periodogram scratch: [n_det][n_seg][NBIN] doubles, n_det * n_seg <= kMaxPeriodograms (4.2 MB)
-static __device__ __align__(256) double g_noalloc_periodograms[kMaxPeriodograms * NBIN];
+// periodogram scratch: [n_det][n_seg] rows, n_det * n_seg <= kMaxPeriodograms (2.1 MB)
+static __device__ __align__(256) float g_noalloc_periodograms[kMaxPeriodograms * (NBIN + 3)];
 
 struct DeviceState {
     bool ready = false;
-    double *scratch = nullptr;
+    float *scratch = nullptr;
 };
 
 DeviceState g_dev[kMaxDevices];
@@ -39,7 +39,7 @@ int setup(int dev, DeviceState **out) {
     if (!s.ready) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_noalloc_periodograms) != cudaSuccess) return AFG_ERR_CUDA;
-        s.scratch = static_cast<double *>(p);
+        s.scratch = static_cast<float *>(p);
         if (prepare_psd_kernels() != cudaSuccess) return AFG_ERR_CUDA;
         s.ready = true;
     }

@@ -590,7 +590,7 @@ extern "C" int afg_stream_start(afg_ctx *ctx, const afg_stream_params *p) {
     void *tmp = nullptr;
     const int64_t K = (p->psd_len - NFFT) / hop + 1;
     E->rb_rows = 2 * std::min(p->max_streams, 16);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, (size_t)E->rb_rows * K * NBIN * sizeof(double), &tmp);
+    if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, periodogram_bytes(E->rb_rows * K), &tmp);
     if (!rc && (cudaMalloc(&E->d_rf_psd, (size_t)E->rb_rows * NBIN * sizeof(double)) != cudaSuccess ||
                 cudaMalloc(&E->d_rf_gains, (size_t)E->rb_rows * NBIN * sizeof(float)) != cudaSuccess)) {
         cudaGetLastError();

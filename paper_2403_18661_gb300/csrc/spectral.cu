@@ -7,10 +7,11 @@
 //                     shared memory (radix-16 passes, fft16.cuh), the window
 //                     applied to the spectrum (a three-bin convolution),
 //                     |X_k|^2 formed in FP32 after an exact power-of-two
-//                     scaling of the segment's spectrum, stored in FP64
-//   k_psd_mean        FP64 mean over the K segments of each epoch (a sliding
-//                     sum over a run of epochs per thread), density scaling
-//                     and one-sided doubling
+//                     scaling of the segment's spectrum, stored as FP32 with
+//                     the segment's exponent
+//   k_psd_mean        sum over the K segments of each epoch in pairs of floats
+//                     (FP64 where segments are too many or too far apart),
+//                     a run of epochs per thread
 //   k_whiten          one 8192-output overlap-save block per CTA: FP32 real
 //                     FFT of 8192 + F - 1 samples (zero padded to NFFT),
 //                     multiply by the epoch's gains, inverse FFT, keep the
@@ -82,8 +83,12 @@ __device__ __forceinline__ void welch_mid_task(float2 *d, int j) {
 // The periodic Hann window is applied in the frequency domain: its DFT has three non-zero bins,
 // so the windowed spectrum is X_k = U_k / 2 - (U_{k-1} + U_{k+1}) / 4 with U the spectrum of the
 // unwindowed segment (U_{-1} = conj U_1, U_{NC+1} = conj U_{NC-1} for a real segment).
+// Row of a segment: P[k] for k <= NC, to be read as P[k] 2^e with e an integer in slot PER_EXP.
+// (PER_ZERO: a segment of zeros.)
+constexpr int PER_EXP = NBIN, PER_ROW = NBIN + 3, PER_ZERO = -(1 << 30);
+
 __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restrict__ x, int64_t x_stride, int hop,
-                                                             double *__restrict__ P, int64_t n_seg,
+                                                             float *__restrict__ P, int64_t n_seg,
                                                              const float *const *__restrict__ rows, float scale) {
     using namespace r16;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -126,7 +131,7 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
     if (t == NT - 1) welch_mid_task(d, 2048);
     __syncthreads();
     // windowed bins k = t + 512 m (and NC) in registers, and the largest component magnitude of the block
-    double *out = P + ((int64_t)det * n_seg + g) * NBIN;
+    float *out = P + ((int64_t)det * n_seg + g) * PER_ROW;
     auto U = [&](int k) -> float2 {
         if (k < 0) return conj(d[pad(-k)]);
         if (k == NC) return *u_nyq;
@@ -160,71 +165,151 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
     // |X_k|^2 = 2^-2s ((2^s X.re)^2 + (2^s X.im)^2): the power-of-two scale is exact and brings the largest
     // component near 2^40, so the FP32 squares neither overflow nor underflow (strain spectra sit near
     // 1e-19, whose squares are below FP32's range); the sum is rounded once in FP32 (relative 1.2e-7, far
-    // below the FP32 transform's own error) and rebuilt as the double with the exponent lowered by 2s, bit
-    // by bit, so no FP64 instruction runs here (the mean over segments is FP64).  NaN and infinity pass through.
+    // below the FP32 transform's own error) and stored as it is, with the exponent -2s in the row: half the
+    // bytes of the double it stands for.  NaN and infinity pass through.
     int e = 0;
     frexpf(mx, &e);
     const int sc = min(40 - e, 120);
     const float s2 = __int_as_float((127 + sc) << 23);  // 2^sc (sc >= -88)
-    const int ebias = 896 - 2 * sc;
-    // c_k scale |X_k|^2 (the density scale and one-sided doubling of the mean, applied here in FP32 so
-    // that the mean over segments is a plain FP64 sum)
-    auto p2 = [&](float2 q, float f) -> double {
-        const float a = q.x * s2, b = q.y * s2;
-        const uint32_t u = __float_as_uint(fmaf(b, b, a * a) * f);
-        const uint32_t E = u >> 23, m23 = u & 0x7FFFFFu;
-        if (E == 0) return 0.0;  // zero (or below 2^-126 of the scaled range)
-        if (E == 255) return __hiloint2double((int)(0x7FF00000u | (m23 ? 0x80000u : 0u)), 0);
-        return __hiloint2double((int)((uint32_t)((int)E + ebias) << 20 | (m23 >> 3)), (int)((m23 & 7u) << 29));
+    // c_k scale |X_k|^2 (the density scale and one-sided doubling of the mean, applied here so that the mean
+    // over segments is a plain sum)
+    auto p2 = [&](float2 q, float f) {
+        const float a = q.x * s2, b = q.y * s2, u = fmaf(b, b, a * a) * f;
+        return u < 0x1p-126f ? 0.f : u;  // zero (or below 2^-126 of the scaled range); NaN stays
     };
     const float f2 = 2.0f * scale;
 #pragma unroll
     for (int m = 0; m < 16; ++m) out[t + NT * m] = p2(X[m], (t | m) ? f2 : scale);
-    if (t == NT - 1) out[NC] = p2(Xn, scale);
-}
-
-// Epochs e0 .. e0 + PSD_EPT - 1 (those below n_psd) of one bin for a fixed segment step SS and count KK:
-// with the running prefix Q[n] of the run's segments (Q[0] = 0), epoch e0 + i is Q[i SS + KK] - Q[i SS];
-// the prefix passes Q[i SS] before it reaches Q[i SS + KK], so those values wait in registers.  One FP64
-// add per segment and one per epoch, every periodogram value of the run loaded once.
-template <int SS, int KK>
-__device__ __forceinline__ void psd_run_fixed(const double *src, double *dst, int64_t e0, int64_t n_psd) {
-    constexpr int E = PSD_EPT, NMAX = (E - 1) * SS + KK;
-    const int n_e = (int)min((int64_t)E, n_psd - e0);
-    const int n_used = (n_e - 1) * SS + KK;
-    const double *s0 = src + e0 * SS * NBIN;
-    double trail[E];
-    double q = 0.0;
-#pragma unroll
-    for (int n = 0; n <= NMAX; ++n) {
-        if (n % SS == 0 && n / SS < E) trail[n / SS] = q;
-        if (n >= KK && (n - KK) % SS == 0 && (n - KK) / SS < n_e) dst[(e0 + (n - KK) / SS) * NBIN] = q - trail[(n - KK) / SS];
-        if (n < NMAX && n < n_used) q += s0[(int64_t)n * NBIN];
+    if (t == NT - 1) {
+        out[NC] = p2(Xn, scale);
+        out[PER_EXP] = __int_as_float(mx == 0.f ? PER_ZERO : -2 * sc);
     }
 }
 
-// grid (ceil(NBIN/256), ceil(n_psd/PSD_EPT), n_det): bin k of epochs [e0, e0 + PSD_EPT) as FP64 sums of the
-// periodograms (already scaled by the density factor; epoch e sums segments [e seg_step, e seg_step + K)):
-// a running prefix for the 8 s epochs of 64 s PSDs at 50 % overlap (step 2, 15 segments), else a sliding sum
-__global__ void k_psd_mean(const double *__restrict__ P, int64_t n_seg, int seg_step, int K,
-                           double *__restrict__ psd, int64_t n_psd) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= NBIN) return;
+// The double u 2^e, bit by bit (no FP64 instruction); u zero, normal, infinite or NaN.
+__device__ __forceinline__ double scaled_double(float v, int e) {
+    const uint32_t u = __float_as_uint(v), E = u >> 23, m23 = u & 0x7FFFFFu;
+    if (E == 0) return 0.0;
+    if (E == 255) return __hiloint2double((int)(0x7FF00000u | (m23 ? 0x80000u : 0u)), 0);
+    return __hiloint2double((int)((uint32_t)((int)E + 896 + e) << 20 | (m23 >> 3)), (int)((m23 & 7u) << 29));
+}
+
+// A sum of non-negative floats as h + l (l a few roundings of h at most)
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ Pair padd(Pair a, Pair b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+    return {s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+}
+__device__ __forceinline__ Pair padd(Pair a, float b) {
+    const float s = __fadd_rn(a.h, b), t = __fsub_rn(s, a.h);
+    return {s, __fadd_rn(a.l, __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b, t)))};
+}
+// The double (h + l) 2^e from its bits: the low part as an integer of the high part's last double place.
+__device__ __forceinline__ double pair_double(Pair a, int e) {
+    const float h = __fadd_rn(a.h, a.l), l = __fsub_rn(a.l, __fsub_rn(h, a.h));
+    const uint32_t u = __float_as_uint(h), E = u >> 23;
+    if (E == 0 || E >= 254) return scaled_double(h, e);
+    const int li = __float2int_rn(l * __uint_as_float((254 - E) << 23) * 0x1p52f);  // |l| <= half a place of h: < 2^28
+    unsigned long long m = ((unsigned long long)((u & 0x7FFFFFu) | 0x800000u) << 29) + (long long)li;
+    int ed = (int)E + 896 + e;
+    if (m < (1ull << 52)) {  // h a power of two and l < 0: one binade down
+        m <<= 1;
+        --ed;
+    }
+    return __longlong_as_double((long long)(((unsigned long long)(ed - 1) << 52) + m));
+}
+
+// grid (ceil(NBIN/256), ceil(n_psd/PSD_EPT), n_det): bin k of epochs [e0, e0 + PSD_EPT) as sums of the
+// periodograms (already scaled by the density factor; epoch e sums segments [e seg_step, e seg_step + K)).
+// The sums are pairs of floats over the run's largest exponent (about 46 bits; the terms have 24 and an FP32
+// transform's error) and only the result is a double: this GPU retires 2 FP64 adds a clock and SM, and the FP64
+// prefix sums of the 64 s PSDs kept that pipe 81 % busy.  For those (step 2, 15 segments) an epoch is a tree
+// over shared partial sums: with A_i = P_2i + P_2i+1, B_i = A_i + A_i+1, C_i = B_i + B_i+2, epoch e is
+// C_e + B_e+4 + A_e+6 + P_2e+14, six pair additions.  Other short sums are formed directly; long ones, and runs
+// whose exponents differ by more than 80 (a segment 2^40 times another), slide an FP64 sum.
+constexpr int PSD_SEGS = 512;  // segments of a run the pair sums hold scales for
+
+__global__ void __launch_bounds__(256) k_psd_mean(const float *__restrict__ P, int64_t n_seg, int seg_step, int K,
+                                                  double *__restrict__ psd, int64_t n_psd) {
+    __shared__ float sf[PSD_SEGS];  // 2^(e_s - e_max) of the run's segments
+    __shared__ int elo, ehi;
+    const int tid = threadIdx.x, k = blockIdx.x * 256 + tid;
     const int64_t e0 = (int64_t)blockIdx.y * PSD_EPT;
-    const int det = blockIdx.z;
-    const double *src = P + (int64_t)det * n_seg * NBIN + k;
-    double *dst = psd + (int64_t)det * n_psd * NBIN + k;
-    if (seg_step == 2 && K == 15) {
-        psd_run_fixed<2, 15>(src, dst, e0, n_psd);
+    const int n_e = (int)min((int64_t)PSD_EPT, n_psd - e0);
+    const float *src = P + ((int64_t)blockIdx.z * n_seg + e0 * seg_step) * PER_ROW;
+    double *dst = psd + ((int64_t)blockIdx.z * n_psd + e0) * NBIN + k;
+    const int64_t ns = (int64_t)(n_e - 1) * seg_step + K;
+    bool pairs = K <= 16 && ns <= PSD_SEGS;
+    if (pairs) {
+        if (tid == 0) {
+            elo = 1 << 20;
+            ehi = -(1 << 20);
+        }
+        __syncthreads();
+        for (int s = tid; s < ns; s += 256) {
+            const int e = __float_as_int(src[(int64_t)s * PER_ROW + PER_EXP]);
+            if (e == PER_ZERO) continue;
+            atomicMin(&elo, e);
+            atomicMax(&ehi, e);
+        }
+        __syncthreads();
+        pairs = ehi - elo <= 80;
+        if (pairs)
+            for (int s = tid; s < ns; s += 256) {
+                const int e = __float_as_int(src[(int64_t)s * PER_ROW + PER_EXP]);
+                sf[s] = e == PER_ZERO ? 0.f : __int_as_float((127 + e - ehi) << 23);
+            }
+        __syncthreads();
+    }
+    if (k >= NBIN) return;
+    src += k;
+    if (pairs && seg_step == 2 && K == 15) {
+        auto at = [&](int s) { return s < ns ? src[(int64_t)s * PER_ROW] * sf[s] : 0.f; };
+        Pair a1 = {0.f, 0.f}, b1 = a1, b2 = a1, c1 = a1, c2 = a1, c3 = a1;  // A_i-1, B_i-1 .., C_i-4 ..
+        float p = at(0);
+#pragma unroll 6
+        for (int i = 0; i < PSD_EPT + 6; ++i) {
+            if (i >= n_e + 6) break;
+            const Pair a = padd(Pair{p, 0.f}, at(2 * i + 1));
+            p = at(2 * i + 2);
+            // the newest A is a = A_i: B_i-1, C_i-3, epoch i - 6
+            const Pair b = padd(a1, a), c = padd(b2, b);
+            if (i >= 6) dst[(int64_t)(i - 6) * NBIN] = pair_double(padd(padd(padd(c3, b1), a), p), ehi);
+            a1 = a;
+            b2 = b1;
+            b1 = b;
+            c3 = c2;
+            c2 = c1;
+            c1 = c;
+        }
         return;
     }
+    if (pairs) {
+        for (int i = 0; i < n_e; ++i) {
+            Pair a = {0.f, 0.f};
+#pragma unroll 5
+            for (int q = 0; q < K; ++q) {
+                const int s = i * seg_step + q;
+                a = padd(a, src[(int64_t)s * PER_ROW] * sf[s]);
+            }
+            dst[(int64_t)i * NBIN] = pair_double(a, ehi);
+        }
+        return;
+    }
+    auto val = [&](int64_t s) {
+        const float *r = src + s * PER_ROW;
+        return scaled_double(r[0], __float_as_int(r[PER_EXP - k]));
+    };
     double acc = 0.0;
-    for (int q = 0; q < K; ++q) acc += src[(e0 * seg_step + q) * NBIN];
-    dst[e0 * NBIN] = acc;
-    for (int64_t e = e0 + 1; e < e0 + PSD_EPT && e < n_psd; ++e) {
-        const int64_t s_old = (e - 1) * seg_step, s_new = s_old + K;
-        for (int q = 0; q < seg_step; ++q) acc += src[(s_new + q) * NBIN] - src[(s_old + q) * NBIN];
-        dst[e * NBIN] = acc;
+    for (int q = 0; q < K; ++q) acc += val(q);
+    dst[0] = acc;
+    for (int64_t i = 1; i < n_e; ++i) {
+        const int64_t s_old = (i - 1) * seg_step, s_new = s_old + K;
+        for (int q = 0; q < seg_step; ++q) acc += val(s_new + q) - val(s_old + q);
+        dst[i * NBIN] = acc;
     }
 }
 
@@ -629,19 +714,19 @@ int launch_psd(afg_ctx *ctx, const float *x, int64_t n, int n_det, int64_t n_psd
     const int64_t K = (psd_span - NFFT) / hop + 1;
     const int64_t seg_step = n_psd > 1 ? psd_step / hop : 0;
     const int64_t n_seg = (n_psd - 1) * seg_step + K;
-    double *P = nullptr;
-    int rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, (size_t)n_det * n_seg * NBIN * sizeof(double), (void **)&P);
+    float *P = nullptr;
+    int rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, periodogram_bytes(n_det * n_seg), (void **)&P);
     if (rc) return rc;
     if (n_seg > 0x7fffffff) return afg_fail(ctx, AFG_ERR_ARG, "psd_estimate: too many segments");
     {
-        // one read of every segment, one FP64 periodogram written per segment
-        KScope ks(ctx, st, KK_PERIODOGRAM, 0.0, (double)n_det * n_seg * (NFFT * 4.0 + NBIN * 8.0));
+        // one read of every segment, one periodogram written per segment
+        KScope ks(ctx, st, KK_PERIODOGRAM, 0.0, (double)n_det * n_seg * (NFFT * 4.0 + NBIN * 4.0));
         k_periodogram<<<dim3((unsigned)n_seg, n_det), r16::NT, WELCH_SMEM, st>>>(x, x_stride, hop, P, n_seg, nullptr,
                                                                                  psd_scale(K, ctx->cfg.fs));
     }
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
-        KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_det * (n_seg + n_psd) * NBIN * 8.0);
+        KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_det * (n_seg * 4.0 + n_psd * 8.0) * NBIN);
         k_psd_mean<<<dim3((NBIN + 255) / 256, (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), 256, 0, st>>>(
             P, n_seg, (int)seg_step, (int)K, psd, n_psd);
     }
@@ -698,17 +783,17 @@ int launch_psd_rows(afg_ctx *ctx, const float *const *rows_dev, int n_rows, int6
     if (n_rows <= 0) return AFG_OK;
     const int hop = ctx->cfg.hop;
     const int64_t K = (psd_span - NFFT) / hop + 1;
-    double *P = nullptr;
-    int rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, (size_t)n_rows * K * NBIN * sizeof(double), (void **)&P);
+    float *P = nullptr;
+    int rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, periodogram_bytes(n_rows * K), (void **)&P);
     if (rc) return rc;
     {
-        KScope ks(ctx, st, KK_PERIODOGRAM, 0.0, (double)n_rows * K * (NFFT * 4.0 + NBIN * 8.0));
+        KScope ks(ctx, st, KK_PERIODOGRAM, 0.0, (double)n_rows * K * (NFFT * 4.0 + NBIN * 4.0));
         k_periodogram<<<dim3((unsigned)K, (unsigned)n_rows), r16::NT, WELCH_SMEM, st>>>(nullptr, 0, hop, P, K,
                                                                                         rows_dev, psd_scale(K, ctx->cfg.fs));
     }
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
-        KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_rows * (K + 1) * NBIN * 8.0);
+        KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_rows * (K * 4.0 + 8.0) * NBIN);
         k_psd_mean<<<dim3((NBIN + 255) / 256, 1, (unsigned)n_rows), 256, 0, st>>>(P, K, 0, (int)K, psd, 1);
     }
     AFG_LAUNCH_CHECK(ctx, "k_psd_mean");
@@ -744,9 +829,9 @@ int launch_whiten_multi(afg_ctx *ctx, const WhitenPiece *pieces_dev, int n_piece
 }
 
 // The Welch kernels on caller-provided scratch and twiddles (no workspace,
-// no context, no accounting).  P must hold n_det * n_seg * NBIN doubles.
+// no context, no accounting).  P must hold periodogram_bytes(n_det * n_seg).
 cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, int64_t psd_step, int64_t psd_span,
-                          int hop, int fs, double *P, double *psd, cudaStream_t st) {
+                          int hop, int fs, float *P, double *psd, cudaStream_t st) {
     const int64_t K = (psd_span - NFFT) / hop + 1;
     const int64_t seg_step = n_psd > 1 ? psd_step / hop : 0;
     const int64_t n_seg = (n_psd - 1) * seg_step + K;

@@ -1,0 +1,38 @@
+"""The Welch average's sums (pairs of floats, or FP64) against the same segments' single periodograms summed in
+float64 on the host: every epoch layout's branch, run boundaries, silent segments and segments far apart in power."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2403_18661_gb300 import abi, inputs  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+NFFT, HOP = 16384, 8192
+# the density factor 1 / (K ...) and its product with |X|^2 are rounded to FP32 on both sides: 4 x 2^-24
+RTOL = 4 * 2.0 ** -24
+
+
+# segments an epoch averages, segments from one epoch to the next: the 64 s PSDs' tree, direct pair sums, long sums
+@pytest.mark.parametrize("k_seg,seg_step", [(15, 2), (15, 1), (4, 3), (16, 16), (1, 2), (31, 2)])
+@pytest.mark.parametrize("kind", ["strain", "silent", "loud"])
+@pytest.mark.parametrize("n_psd", [1, 32, 45])
+def test_epoch_sums_match_single_periodograms(k_seg, seg_step, kind, n_psd):
+    n_seg = (n_psd - 1) * seg_step + k_seg
+    n = (n_seg - 1) * HOP + NFFT
+    rng = np.random.default_rng(n_seg)
+    x = (1e-21 * rng.standard_normal((2, n))).astype(np.float32)
+    if kind == "silent":
+        x[0, :5 * HOP] = 0.0
+        x[1, n // 2:n // 2 + 3 * HOP] = 0.0
+    if kind == "loud":  # the last segment: 2^100 times the others in power
+        x[:, -HOP:] *= np.float32(2.0 ** 50)
+    wl = inputs.PLAIN_64S
+    ctx = abi.Context(wl, inputs.make_weights(wl.net, 1))
+    xd = torch.from_numpy(x).cuda()
+    one = ctx.psd_estimate(xd, n_psd=n_seg, psd_step=HOP, psd_span=NFFT).cpu().numpy()
+    got = ctx.psd_estimate(xd, n_psd=n_psd, psd_step=seg_step * HOP, psd_span=(k_seg - 1) * HOP + NFFT).cpu().numpy()
+    want = np.stack([one[:, e * seg_step:e * seg_step + k_seg].mean(axis=1) for e in range(n_psd)], axis=1)
+    assert np.all(np.abs(got - want) <= RTOL * want)
+    ctx.close()
