@@ -4,12 +4,15 @@
 //
 // The background statistics are sorted in decreasing order on the device by an
 // LSD radix sort of order-preserving 32-bit keys (4 passes of 8 bits, each pass
-// stable: per-tile digit histograms, one exclusive scan over (digit, tile), and a
-// scatter that ranks equal digits in input order).  Launches are sized by the
+// stable: per-tile digit histograms, a scan of each digit's row over the tiles, and a
+// scatter that adds up the digits before and ranks equal digits in input order).  The
+// first pass reads the statistics, the last writes them.  Launches are sized by the
 // capacity; only the tiles that hold keys do work.  Each foreground statistic x
-// then gets count = #{background > x} by binary search, and FAR = count / livetime.
+// then gets count = #{background > x} by a 32-way search (one warp), and FAR = count / livetime.
 // The background count may live on the device (as afg_batch_run writes it), so
 // every kernel reads n = min(*n_dev, cap) itself and nothing synchronises.
+// A handful of small kernels in a row: latency sets the time (0.93 million events: 330 us with the histogram
+// scanned by one block (43 us of each pass) and four barriers per 256 keys of the scatter, 95 us now).
 #include <stdint.h>
 
 #include <algorithm>
@@ -41,20 +44,23 @@ __device__ __forceinline__ float value_of(uint32_t k) {
     return __uint_as_float(b);
 }
 
-__global__ void k_far_keys(const float *__restrict__ stat, const int64_t *__restrict__ idx, const int64_t *n_dev,
-                           int64_t cap, uint32_t *__restrict__ keys) {
-    const int64_t n = dev_count(n_dev, cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = key_of(stat[idx ? idx[i] : i]);
-}
-
 // tiles that hold keys
 __device__ __forceinline__ int occupied_tiles(int64_t n) { return (int)((n + RS_TILE - 1) / RS_TILE); }
 
+// The keys a pass reads: of the previous pass, or (keys null, first pass) of the statistics.
+struct KeySource {
+    const uint32_t *keys;
+    const float *stat;
+    const int64_t *idx;
+    __device__ __forceinline__ uint32_t operator()(int64_t i) const {
+        return keys ? keys[i] : key_of(stat[idx ? idx[i] : i]);
+    }
+};
+
 // hist[d * n_eff + tile] = keys of the tile whose digit (at `shift`) is d, over the
 // n_eff = ceil(n / RS_TILE) tiles that hold keys (blocks past them return at once)
-__global__ void __launch_bounds__(RS_T) k_rs_hist(const uint32_t *__restrict__ keys, const int64_t *n_dev,
-                                                  int64_t cap, int shift, uint32_t *__restrict__ hist) {
+__global__ void __launch_bounds__(RS_T) k_rs_hist(const KeySource src, const int64_t *n_dev, int64_t cap, int shift,
+                                                  uint32_t *__restrict__ hist) {
     __shared__ uint32_t h[256];
     const int64_t n = dev_count(n_dev, cap);
     const int n_eff = occupied_tiles(n);
@@ -62,127 +68,140 @@ __global__ void __launch_bounds__(RS_T) k_rs_hist(const uint32_t *__restrict__ k
     h[threadIdx.x] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    uint32_t k[RS_ROUNDS];
+#pragma unroll
     for (int r = 0; r < RS_ROUNDS; ++r) {
         const int64_t i = base + r * RS_T + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
+        k[r] = i < n ? src(i) : 0u;
     }
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r)
+        if (base + r * RS_T + threadIdx.x < n) atomicAdd(&h[(k[r] >> shift) & 255u], 1u);
     __syncthreads();
     hist[(size_t)threadIdx.x * n_eff + blockIdx.x] = h[threadIdx.x];
 }
 
-// In-place exclusive scan of the 256 n_eff histogram entries (digit-major, so the scan
-// order is (digit, tile)), one block walking chunks of 1024 with a running carry.  Each
-// chunk: a warp scan, the 32 warp totals through shared memory (double-buffered, so one
-// barrier per chunk), and every warp scans those totals itself.  Loads run SCAN_AHEAD
-// chunks ahead of the chunk being scanned.
-constexpr int SCAN_AHEAD = 4;
-__global__ void __launch_bounds__(1024) k_rs_scan(uint32_t *__restrict__ a, const int64_t *n_dev, int64_t cap) {
-    __shared__ uint32_t wsum[2][32];
-    const int64_t n = dev_count(n_dev, cap);
-    const int64_t m = (int64_t)256 * occupied_tiles(n);
+// grid (256): exclusive scan of digit d's row of n_eff tile counts in place, and its sum to total[d]
+__global__ void __launch_bounds__(256) k_rs_scan(uint32_t *__restrict__ hist, const int64_t *n_dev, int64_t cap,
+                                                 uint32_t *__restrict__ total) {
+    __shared__ uint32_t wsum[2][8];
+    const int n_eff = occupied_tiles(dev_count(n_dev, cap));
+    uint32_t *a = hist + (size_t)blockIdx.x * n_eff;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    uint32_t v[SCAN_AHEAD];
-#pragma unroll
-    for (int k = 0; k < SCAN_AHEAD; ++k) {
-        const int64_t i = (int64_t)k * 1024 + t;
-        v[k] = i < m ? a[i] : 0u;
-    }
     uint32_t carry = 0;
     int buf = 0;
-    for (int64_t c0 = 0; c0 < m; c0 += 1024 * SCAN_AHEAD) {
-        uint32_t nxt[SCAN_AHEAD];
+    for (int c0 = 0; c0 < n_eff; c0 += 1024, buf ^= 1) {  // four consecutive entries a thread
+        uint32_t v[4], x = 0;
 #pragma unroll
-        for (int k = 0; k < SCAN_AHEAD; ++k) {
-            const int64_t i = c0 + (int64_t)(SCAN_AHEAD + k) * 1024 + t;
-            nxt[k] = i < m ? a[i] : 0u;
+        for (int k = 0; k < 4; ++k) {
+            const int i = c0 + 4 * t + k;
+            v[k] = i < n_eff ? a[i] : 0u;
+            x += v[k];
+        }
+        const uint32_t own = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[buf][warp] = x;
+        __syncthreads();
+        uint32_t before = carry + x - own;
+        for (int w = 0; w < 8; ++w) {
+            const uint32_t s = wsum[buf][w];
+            if (w < warp) before += s;
+            carry += s;
         }
 #pragma unroll
-        for (int k = 0; k < SCAN_AHEAD; ++k) {
-            uint32_t x = v[k];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (lane == 31) wsum[buf][warp] = x;
-            __syncthreads();
-            uint32_t w = wsum[buf][lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            const uint32_t before = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
-            const uint32_t total = __shfl_sync(0xffffffffu, w, 31);
-            const int64_t i = c0 + (int64_t)k * 1024 + t;
-            if (i < m) a[i] = carry + (warp ? before : 0u) + x - v[k];
-            carry += total;
-            buf ^= 1;
+        for (int k = 0; k < 4; ++k) {
+            const int i = c0 + 4 * t + k;
+            if (i < n_eff) a[i] = before;
+            before += v[k];
         }
-#pragma unroll
-        for (int k = 0; k < SCAN_AHEAD; ++k) v[k] = nxt[k];
     }
+    if (t == 0) total[blockIdx.x] = carry;
 }
 
-// Stable scatter of one tile: key index base + r * RS_T + t is processed in round r by
-// thread t, so (round, thread) order is input order; inside a round, equal digits are
-// ranked by warp (lower warps first) and by lane (match_any peers with lower lanes).
-__global__ void __launch_bounds__(RS_T) k_rs_scatter(const uint32_t *__restrict__ kin, uint32_t *__restrict__ kout,
-                                                     const int64_t *n_dev, int64_t cap, int shift,
-                                                     const uint32_t *__restrict__ hist) {
-    __shared__ uint32_t running[256];          // keys of each digit placed by earlier rounds (+ tile base)
-    __shared__ uint32_t wcnt[RS_WARPS][257];   // per-warp digit counts of the current round
+// Stable scatter of one tile: warp w takes its 32 RS_ROUNDS consecutive keys, 32 a round; equal digits of a round
+// are ranked by lane (match_any peers with lower lanes) behind the warp's count so far, then the warps' counts are
+// added up per digit.  Writes keys, or (last pass, out set) the statistics themselves.
+__global__ void __launch_bounds__(RS_T) k_rs_scatter(const KeySource src, uint32_t *__restrict__ kout,
+                                                     float *__restrict__ out, const int64_t *n_dev, int64_t cap, int shift,
+                                                     const uint32_t *__restrict__ hist,
+                                                     const uint32_t *__restrict__ total) {
+    __shared__ uint32_t wcnt[RS_WARPS][257];  // per-warp digit counts, then each warp's first place
+    __shared__ uint32_t dsum[RS_WARPS];
     const int64_t n = dev_count(n_dev, cap);
     const int n_eff = occupied_tiles(n);
     if ((int)blockIdx.x >= n_eff) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    running[t] = hist[(size_t)t * n_eff + blockIdx.x];
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        for (int i = t; i < RS_WARPS * 257; i += RS_T) (&wcnt[0][0])[i] = 0;
-        __syncthreads();
-        const int64_t i = base + r * RS_T + t;
-        const bool valid = i < n;
-        const uint32_t key = valid ? kin[i] : 0u;
-        const uint32_t d = valid ? ((key >> shift) & 255u) : 256u;  // 256: no key
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t rank = __popc(peers & lt);
-        if (rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        uint32_t before = 0;  // same-digit keys of lower warps in this round
-        for (int w = 0; w < warp; ++w) before += wcnt[w][d];
-        if (valid) kout[running[d] + before + rank] = key;
-        __syncthreads();
-        uint32_t tot = 0;  // thread t advances digit t
-        for (int w = 0; w < RS_WARPS; ++w) tot += wcnt[w][t];
-        running[t] += tot;
-        __syncthreads();
+    for (int i = lane; i < 257; i += 32) wcnt[warp][i] = 0;
+    // keys of lower digits: exclusive sum of the 256 totals (thread t: digit t)
+    const uint32_t dt = total[t];
+    uint32_t x = dt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
     }
+    if (lane == 31) dsum[warp] = x;
+    uint32_t place = x - dt + hist[(size_t)t * n_eff + blockIdx.x];
+    const int64_t base = (int64_t)blockIdx.x * RS_TILE + warp * (32 * RS_ROUNDS) + lane;
+    uint32_t key[RS_ROUNDS], rank[RS_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) key[r] = base + 32 * r < n ? src(base + 32 * r) : 0u;
+    const uint32_t lt = (1u << lane) - 1u;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        const uint32_t d = base + 32 * r < n ? (key[r] >> shift) & 255u : 256u;  // 256: no key
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        rank[r] = wcnt[warp][d] + __popc(peers & lt);
+        __syncwarp();
+        if ((peers & lt) == 0) wcnt[warp][d] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) place += dsum[w];
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {  // thread t: digit t
+        const uint32_t c = wcnt[w][t];
+        wcnt[w][t] = place;
+        place += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r)
+        if (base + 32 * r < n) {
+            const uint32_t p = wcnt[warp][(key[r] >> shift) & 255u] + rank[r];
+            if (out) out[p] = value_of(key[r]);
+            else kout[p] = key[r];
+        }
 }
 
-__global__ void k_far_values(const uint32_t *__restrict__ keys, const int64_t *n_dev, int64_t cap,
-                             float *__restrict__ sorted) {
-    const int64_t n = dev_count(n_dev, cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        sorted[i] = value_of(keys[i]);
-}
-
-// count = #{sorted > x}: the first index whose value is <= x in the decreasing array
+// count = #{sorted > x}: the first index whose value is <= x in the decreasing array.  One warp per x: each step
+// splits the range in 33 at 32 probes.
 __global__ void k_far_count(const float *__restrict__ sorted, const int64_t *n_dev, int64_t cap,
                             const float *__restrict__ fg, int64_t n_fg, double livetime, int64_t *__restrict__ n_above,
                             double *__restrict__ far) {
     const int64_t n = dev_count(n_dev, cap);
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_fg; j += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; j < n_fg; j += warps) {
         const float x = fg[j];
-        int64_t lo = 0, hi = n;
+        int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
         while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (sorted[mid] > x) lo = mid + 1;
-            else hi = mid;
+            const int64_t step = (hi - lo + 32) / 33, i = lo + step * (lane + 1) - 1;  // probes, in order
+            const uint32_t above = __ballot_sync(0xffffffffu, i < hi && sorted[i] > x);
+            const int c = __popc(above);  // the first c probes are above x
+            const int64_t nhi = lo + step * (c + 1) - 1;
+            lo += step * c;
+            hi = c < 32 && nhi < hi ? nhi : hi;
         }
-        if (n_above) n_above[j] = lo;
-        if (far) far[j] = (double)lo / livetime;
+        if (lane == 0) {
+            if (n_above) n_above[j] = lo;
+            if (far) far[j] = (double)lo / livetime;
+        }
     }
 }
 
@@ -192,7 +211,7 @@ int launch_far(afg_ctx *ctx, const float *bg_stat, const int64_t *bg_idx, const 
                double livetime_s, const float *fg, int64_t n_fg, int64_t *n_above, double *far, float *bg_sorted,
                cudaStream_t st) {
     const int n_tiles = (int)std::max<int64_t>(1, (bg_cap + RS_TILE - 1) / RS_TILE);
-    const int64_t m = (int64_t)256 * n_tiles;
+    const int64_t m = (int64_t)256 * n_tiles + 256;  // and the digits' totals
     void *wk = nullptr, *wh = nullptr, *ws = nullptr;
     int rc = afg_ws_reserve(ctx, WS_FAR_KEYS, (size_t)2 * std::max<int64_t>(bg_cap, 1) * sizeof(uint32_t), &wk);
     if (!rc) rc = afg_ws_reserve(ctx, WS_FAR_HIST, (size_t)m * sizeof(uint32_t), &wh);
@@ -203,19 +222,20 @@ int launch_far(afg_ctx *ctx, const float *bg_stat, const int64_t *bg_idx, const 
     if (rc) return rc;
     uint32_t *ka = static_cast<uint32_t *>(wk), *kb = ka + std::max<int64_t>(bg_cap, 1);
     uint32_t *hist = static_cast<uint32_t *>(wh);
-    const unsigned g1 = (unsigned)std::min<int64_t>((bg_cap + 255) / 256 + 1, 152 * 16);
+    uint32_t *total = hist + (int64_t)256 * n_tiles;
     {
         KScope ks(ctx, st, KK_FAR, 0.0, (double)bg_cap * (4.0 + 8.0 + 4.0 * 4 * 4 + 4.0) + n_fg * 20.0);
-        k_far_keys<<<g1, 256, 0, st>>>(bg_stat, bg_idx, n_bg_dev, bg_cap, ka);
+        KeySource src = {nullptr, bg_stat, bg_idx};
         for (int pass = 0; pass < 4; ++pass) {
-            k_rs_hist<<<n_tiles, RS_T, 0, st>>>(ka, n_bg_dev, bg_cap, 8 * pass, hist);
-            k_rs_scan<<<1, 1024, 0, st>>>(hist, n_bg_dev, bg_cap);
-            k_rs_scatter<<<n_tiles, RS_T, 0, st>>>(ka, kb, n_bg_dev, bg_cap, 8 * pass, hist);
+            k_rs_hist<<<n_tiles, RS_T, 0, st>>>(src, n_bg_dev, bg_cap, 8 * pass, hist);
+            k_rs_scan<<<256, 256, 0, st>>>(hist, n_bg_dev, bg_cap, total);
+            k_rs_scatter<<<n_tiles, RS_T, 0, st>>>(src, ka, pass == 3 ? bg_sorted : nullptr, n_bg_dev, bg_cap, 8 * pass,
+                                                   hist, total);
+            src.keys = ka;
             std::swap(ka, kb);
         }
-        k_far_values<<<g1, 256, 0, st>>>(ka, n_bg_dev, bg_cap, bg_sorted);
         if (n_fg > 0)
-            k_far_count<<<(unsigned)std::min<int64_t>((n_fg + 255) / 256, 152 * 16), 256, 0, st>>>(
+            k_far_count<<<(unsigned)std::min<int64_t>((n_fg + 7) / 8, 152 * 16), 256, 0, st>>>(
                 bg_sorted, n_bg_dev, bg_cap, fg, n_fg, livetime_s, n_above, far);
     }
     AFG_LAUNCH_CHECK(ctx, "far (radix sort + rank count)");
