@@ -162,6 +162,7 @@ enum KernelKind {
     KK_FAR,
     KK_RESAMPLE,
     KK_CONV_SPLIT,
+    KK_TINY32,
     KK_COUNT
 };
 extern const char *const kKernelNames[KK_COUNT];
@@ -335,6 +336,10 @@ int launch_infer_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_strid
                       int64_t stride, int64_t n_win, int64_t shift, float *logits, cudaStream_t st);
 int launch_stem_gn_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first, int64_t stride,
                         int64_t shift, int64_t w0, int nw, float *f0, float *f1, cudaStream_t st);
+// net_tiny32.cu
+bool net_tiny32_fits(const afg_ctx *ctx);
+int launch_infer_tiny32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stride, int64_t first, int64_t stride,
+                        int64_t n_win, int64_t shift, float *logits, cudaStream_t st);
 // net_split.cu
 int net_split_prepare(afg_ctx *ctx);
 void net_split_release(afg_ctx *ctx);

@@ -10,7 +10,8 @@
 // strided view of the activation buffer (implicit GEMM, no im2col copy).
 //
 // Networks whose widths are all 64..512 run on the tensor cores instead
-// (net_split.cu); this path serves the others and contexts with a memory budget.
+// (net_split.cu) and the 16-channel one-stage network fused (net_tiny32.cu); this
+// path serves the others, and wide ones in contexts with a memory budget.
 //
 // Per conv: k_conv_fp32 (tiled SIMT GEMM) writes the raw output; then
 // k_groupnorm computes the group statistics of each window (two passes,
@@ -655,6 +656,7 @@ static int64_t simt_chunk(const afg_ctx *ctx, int64_t n_win) {
 // Reserve what launch_infer_fp32 over n_win windows uses (a graph capture allows no allocation).
 int infer_fp32_reserve(afg_ctx *ctx, int64_t n_win) {
     if (net_split_available(ctx)) return net_split_reserve(ctx, n_win);
+    if (net_tiny32_fits(ctx)) return AFG_OK;  // (no workspaces)
     const size_t bytes = (size_t)(simt_chunk(ctx, n_win) * ctx->plan.max_act_per_window) * sizeof(float);
     void *tmp = nullptr;
     int rc = AFG_OK;
@@ -666,6 +668,7 @@ int launch_infer_fp32(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_strid
                       int64_t n_win, int64_t shift, float *logits, cudaStream_t st) {
     if (net_split_available(ctx))
         return launch_infer_split(ctx, y, n_y, y_stride, first, stride, n_win, shift, logits, st);
+    if (net_tiny32_fits(ctx)) return launch_infer_tiny32(ctx, y, n_y, y_stride, first, stride, n_win, shift, logits, st);
     const NetPlan &P = ctx->plan;
     const int G = P.net.groups;
     const float eps = P.net.eps;
