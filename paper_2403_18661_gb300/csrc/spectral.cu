@@ -130,28 +130,29 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
     for (int m = 1; m < 4; ++m) welch_mid_task(d, t + NT * m);
     if (t == NT - 1) welch_mid_task(d, 2048);
     __syncthreads();
-    // windowed bins k = t + 512 m (and NC) in registers, and the largest component magnitude of the block
+    // windowed bins k = 16 t .. 16 t + 15 (and NC) in registers, each spectrum value read once (18 reads a thread; bins
+    // t + 512 m read each value three times, and shared memory is the busiest pipe of this kernel), and the
+    // largest component magnitude of the block
     float *out = P + ((int64_t)det * n_seg + g) * PER_ROW;
-    auto U = [&](int k) -> float2 {
-        if (k < 0) return conj(d[pad(-k)]);
-        if (k == NC) return *u_nyq;
-        if (k > NC) return conj(d[pad(2 * NC - k)]);
-        return d[pad(k)];
-    };
-    auto windowed = [&](int k) {
-        const float2 l = U(k - 1), c = U(k), r = U(k + 1);
-        return make_float2(0.5f * c.x - 0.25f * (l.x + r.x), 0.5f * c.y - 0.25f * (l.y + r.y));
-    };
+    float2 U[18];  // U_{16 t - 1} .. U_{16 t + 16}
+    {
+        const float2 *p = d + pad(16 * t);  // = d + 17 t
+#pragma unroll
+        for (int m = 0; m < 16; ++m) U[m + 1] = p[m];
+        U[0] = t ? p[-2] : conj(U[2]);
+        U[17] = t < NT - 1 ? p[17] : *u_nyq;
+    }
     float2 X[16];
     float mx = 0.f;
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
-        X[m] = windowed(t + NT * m);
+        X[m] = make_float2(0.5f * U[m + 1].x - 0.25f * (U[m].x + U[m + 2].x), 0.5f * U[m + 1].y - 0.25f * (U[m].y + U[m + 2].y));
         mx = fmaxf(mx, fmaxf(fabsf(X[m].x), fabsf(X[m].y)));
     }
     float2 Xn = make_float2(0.f, 0.f);
-    if (t == NT - 1) {
-        Xn = windowed(NC);
+    if (t == NT - 1) {  // bin NC: U_NC + 1 = conj U_NC - 1
+        const float2 r = conj(U[16]);
+        Xn = make_float2(0.5f * U[17].x - 0.25f * (U[16].x + r.x), 0.5f * U[17].y - 0.25f * (U[16].y + r.y));
         mx = fmaxf(mx, fmaxf(fabsf(Xn.x), fabsf(Xn.y)));
     }
 #pragma unroll
@@ -178,8 +179,10 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
         return u < 0x1p-126f ? 0.f : u;  // zero (or below 2^-126 of the scaled range); NaN stays
     };
     const float f2 = 2.0f * scale;
+    float4 *o4 = reinterpret_cast<float4 *>(out + 16 * t);  // (rows are 16-byte aligned)
 #pragma unroll
-    for (int m = 0; m < 16; ++m) out[t + NT * m] = p2(X[m], (t | m) ? f2 : scale);
+    for (int m = 0; m < 4; ++m)
+        o4[m] = make_float4(p2(X[4 * m], (t | m) ? f2 : scale), p2(X[4 * m + 1], f2), p2(X[4 * m + 2], f2), p2(X[4 * m + 3], f2));
     if (t == NT - 1) {
         out[NC] = p2(Xn, scale);
         out[PER_EXP] = __int_as_float(mx == 0.f ? PER_ZERO : -2 * sc);
@@ -194,35 +197,43 @@ __device__ __forceinline__ double scaled_double(float v, int e) {
     return __hiloint2double((int)((uint32_t)((int)E + 896 + e) << 20 | (m23 >> 3)), (int)((m23 & 7u) << 29));
 }
 
-// A sum of non-negative floats as h + l (l a few roundings of h at most)
-struct Pair {
-    float h, l;
+// Two sums of non-negative floats (two bins) as h + l (l a few roundings of h at most), in packed instructions
+struct Pair2 {
+    float2 h, l;
 };
-__device__ __forceinline__ Pair padd(Pair a, Pair b) {
-    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-    return {s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ Pair2 padd(Pair2 a, Pair2 b) {
+    const float2 s = __fadd2_rn(a.h, b.h), t = sub2(s, a.h);
+    const float2 e = __fadd2_rn(sub2(a.h, sub2(s, t)), sub2(b.h, t));
+    return {s, __fadd2_rn(__fadd2_rn(a.l, b.l), e)};
 }
-__device__ __forceinline__ Pair padd(Pair a, float b) {
-    const float s = __fadd_rn(a.h, b), t = __fsub_rn(s, a.h);
-    return {s, __fadd_rn(a.l, __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b, t)))};
+__device__ __forceinline__ Pair2 padd(Pair2 a, float2 b) {
+    const float2 s = __fadd2_rn(a.h, b), t = sub2(s, a.h);
+    return {s, __fadd2_rn(a.l, __fadd2_rn(sub2(a.h, sub2(s, t)), sub2(b, t)))};
+}
+__device__ __forceinline__ Pair2 psum(float2 a, float2 b) {
+    const float2 s = __fadd2_rn(a, b), t = sub2(s, a);
+    return {s, __fadd2_rn(sub2(a, sub2(s, t)), sub2(b, t))};
 }
 // The double (h + l) 2^e from its bits: the low part as an integer of the high part's last double place.
-__device__ __forceinline__ double pair_double(Pair a, int e) {
-    const float h = __fadd_rn(a.h, a.l), l = __fsub_rn(a.l, __fsub_rn(h, a.h));
+__device__ __forceinline__ double pair_double(float ah, float al, int e) {
+    const float h = __fadd_rn(ah, al), l = __fsub_rn(al, __fsub_rn(h, ah));
     const uint32_t u = __float_as_uint(h), E = u >> 23;
-    if (E == 0 || E >= 254) return scaled_double(h, e);
+    if (E - 1u >= 253u) return scaled_double(h, e);  // zero, (nearly) infinite or NaN
     const int li = __float2int_rn(l * __uint_as_float((254 - E) << 23) * 0x1p52f);  // |l| <= half a place of h: < 2^28
-    unsigned long long m = ((unsigned long long)((u & 0x7FFFFFu) | 0x800000u) << 29) + (long long)li;
+    // mantissa 2^52 (1.m) + li in two words
+    uint32_t lo = (u << 29) + (uint32_t)li;
+    uint32_t hi = ((u & 0x7FFFFFu) >> 3) + (uint32_t)(li >> 31) + (lo < (u << 29) ? 1u : 0u);  // (below the leading one)
     int ed = (int)E + 896 + e;
-    if (m < (1ull << 52)) {  // h a power of two and l < 0: one binade down
-        m <<= 1;
+    if (hi >> 31) {  // h a power of two and l < 0: one binade down
+        hi = (((hi + 0x100000u) << 1) | (lo >> 31)) - 0x100000u;
+        lo <<= 1;
         --ed;
     }
-    return __longlong_as_double((long long)(((unsigned long long)(ed - 1) << 52) + m));
+    return __hiloint2double((int)(((uint32_t)ed << 20) + hi), (int)lo);
 }
 
-// grid (ceil(NBIN/256), ceil(n_psd/PSD_EPT), n_det): bin k of epochs [e0, e0 + PSD_EPT) as sums of the
+// grid (ceil(NBIN / 2 PSD_T), ceil(n_psd / PSD_EPT), n_det): the bins of epochs [e0, e0 + PSD_EPT) as sums of the
 // periodograms (already scaled by the density factor; epoch e sums segments [e seg_step, e seg_step + K)).
 // The sums are pairs of floats over the run's largest exponent (about 46 bits; the terms have 24 and an FP32
 // transform's error) and only the result is a double: this GPU retires 2 FP64 adds a clock and SM, and the FP64
@@ -232,11 +243,14 @@ __device__ __forceinline__ double pair_double(Pair a, int e) {
 // whose exponents differ by more than 80 (a segment 2^40 times another), slide an FP64 sum.
 constexpr int PSD_SEGS = 512;  // segments of a run the pair sums hold scales for
 
-__global__ void __launch_bounds__(256) k_psd_mean(const float *__restrict__ P, int64_t n_seg, int seg_step, int K,
-                                                  double *__restrict__ psd, int64_t n_psd) {
+// A thread takes bins k and k + PSD_T as the halves of packed additions (the loads and stores of both coalesce).
+constexpr int PSD_T = 128;
+
+__global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P, int64_t n_seg, int seg_step, int K,
+                                                    double *__restrict__ psd, int64_t n_psd) {
     __shared__ float sf[PSD_SEGS];  // 2^(e_s - e_max) of the run's segments
     __shared__ int elo, ehi;
-    const int tid = threadIdx.x, k = blockIdx.x * 256 + tid;
+    const int tid = threadIdx.x, k = blockIdx.x * 2 * PSD_T + tid;
     const int64_t e0 = (int64_t)blockIdx.y * PSD_EPT;
     const int n_e = (int)min((int64_t)PSD_EPT, n_psd - e0);
     const float *src = P + ((int64_t)blockIdx.z * n_seg + e0 * seg_step) * PER_ROW;
@@ -249,7 +263,7 @@ __global__ void __launch_bounds__(256) k_psd_mean(const float *__restrict__ P, i
             ehi = -(1 << 20);
         }
         __syncthreads();
-        for (int s = tid; s < ns; s += 256) {
+        for (int s = tid; s < ns; s += PSD_T) {
             const int e = __float_as_int(src[(int64_t)s * PER_ROW + PER_EXP]);
             if (e == PER_ZERO) continue;
             atomicMin(&elo, e);
@@ -258,58 +272,87 @@ __global__ void __launch_bounds__(256) k_psd_mean(const float *__restrict__ P, i
         __syncthreads();
         pairs = ehi - elo <= 80;
         if (pairs)
-            for (int s = tid; s < ns; s += 256) {
+            for (int s = tid; s < ns; s += PSD_T) {
                 const int e = __float_as_int(src[(int64_t)s * PER_ROW + PER_EXP]);
                 sf[s] = e == PER_ZERO ? 0.f : __int_as_float((127 + e - ehi) << 23);
             }
         __syncthreads();
     }
+    const bool second = k + PSD_T < NBIN;  // (else the second half repeats the first)
     if (k >= NBIN) return;
+    const int k2 = second ? PSD_T : 0;
     src += k;
+    auto put = [&](int i, Pair2 a) {
+        dst[(int64_t)i * NBIN] = pair_double(a.h.x, a.l.x, ehi);
+        if (second) dst[(int64_t)i * NBIN + PSD_T] = pair_double(a.h.y, a.l.y, ehi);
+    };
+    const float2 zero = make_float2(0.f, 0.f);
     if (pairs && seg_step == 2 && K == 15) {
-        auto at = [&](int s) { return s < ns ? src[(int64_t)s * PER_ROW] * sf[s] : 0.f; };
-        Pair a1 = {0.f, 0.f}, b1 = a1, b2 = a1, c1 = a1, c2 = a1, c3 = a1;  // A_i-1, B_i-1 .., C_i-4 ..
-        float p = at(0);
-#pragma unroll 6
-        for (int i = 0; i < PSD_EPT + 6; ++i) {
-            if (i >= n_e + 6) break;
-            const Pair a = padd(Pair{p, 0.f}, at(2 * i + 1));
-            p = at(2 * i + 2);
-            // the newest A is a = A_i: B_i-1, C_i-3, epoch i - 6
-            const Pair b = padd(a1, a), c = padd(b2, b);
-            if (i >= 6) dst[(int64_t)(i - 6) * NBIN] = pair_double(padd(padd(padd(c3, b1), a), p), ehi);
-            a1 = a;
-            b2 = b1;
-            b1 = b;
-            c3 = c2;
-            c2 = c1;
-            c1 = c;
+        constexpr int ST = 6;  // steps whose loads are in flight together
+        Pair2 a1 = {zero, zero}, b1 = a1, b2 = a1, c1 = a1, c2 = a1, c3 = a1;  // A_i-1, B_i-2 .., C_i-4 ..
+        float2 p = make_float2(src[0] * sf[0], src[k2] * sf[0]);
+        const float *row = src + PER_ROW;
+        for (int i0 = 0; i0 < n_e + 6; i0 += ST, row += 2 * ST * PER_ROW) {
+            float2 q[2 * ST];
+            if (2 * (i0 + ST) < ns) {
+#pragma unroll
+                for (int j = 0; j < 2 * ST; ++j) {
+                    const float f = sf[2 * i0 + 1 + j];
+                    q[j] = make_float2(row[j * PER_ROW] * f, row[j * PER_ROW + k2] * f);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2 * ST; ++j) {
+                    const bool in = 2 * i0 + 1 + j < ns;
+                    const float f = in ? sf[2 * i0 + 1 + j] : 0.f;
+                    q[j] = in ? make_float2(row[j * PER_ROW] * f, row[j * PER_ROW + k2] * f) : zero;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < ST; ++j) {
+                const int i = i0 + j;
+                const Pair2 a = psum(p, q[2 * j]);
+                p = q[2 * j + 1];
+                // the newest A is a = A_i: B_i-1, C_i-3, epoch i - 6
+                const Pair2 b = padd(a1, a), c = padd(b2, b);
+                if (i >= 6 && i < n_e + 6) put(i - 6, padd(padd(padd(c3, b1), a), p));
+                a1 = a;
+                b2 = b1;
+                b1 = b;
+                c3 = c2;
+                c2 = c1;
+                c1 = c;
+            }
         }
         return;
     }
     if (pairs) {
         for (int i = 0; i < n_e; ++i) {
-            Pair a = {0.f, 0.f};
+            Pair2 a = {zero, zero};
 #pragma unroll 5
             for (int q = 0; q < K; ++q) {
                 const int s = i * seg_step + q;
-                a = padd(a, src[(int64_t)s * PER_ROW] * sf[s]);
+                const float *r = src + (int64_t)s * PER_ROW;
+                a = padd(a, make_float2(r[0] * sf[s], r[k2] * sf[s]));
             }
-            dst[(int64_t)i * NBIN] = pair_double(a, ehi);
+            put(i, a);
         }
         return;
     }
-    auto val = [&](int64_t s) {
-        const float *r = src + s * PER_ROW;
-        return scaled_double(r[0], __float_as_int(r[PER_EXP - k]));
-    };
-    double acc = 0.0;
-    for (int q = 0; q < K; ++q) acc += val(q);
-    dst[0] = acc;
-    for (int64_t i = 1; i < n_e; ++i) {
-        const int64_t s_old = (i - 1) * seg_step, s_new = s_old + K;
-        for (int q = 0; q < seg_step; ++q) acc += val(s_new + q) - val(s_old + q);
-        dst[i * NBIN] = acc;
+    for (int h = 0; h < (second ? 2 : 1); ++h) {
+        const int kk = h ? PSD_T : 0;
+        auto val = [&](int64_t s) {
+            const float *r = src + s * PER_ROW;
+            return scaled_double(r[kk], __float_as_int(r[PER_EXP - k]));
+        };
+        double acc = 0.0;
+        for (int q = 0; q < K; ++q) acc += val(q);
+        dst[kk] = acc;
+        for (int64_t i = 1; i < n_e; ++i) {
+            const int64_t s_old = (i - 1) * seg_step, s_new = s_old + K;
+            for (int q = 0; q < seg_step; ++q) acc += val(s_new + q) - val(s_old + q);
+            dst[i * NBIN + kk] = acc;
+        }
     }
 }
 
@@ -727,7 +770,7 @@ int launch_psd(afg_ctx *ctx, const float *x, int64_t n, int n_det, int64_t n_psd
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
         KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_det * (n_seg * 4.0 + n_psd * 8.0) * NBIN);
-        k_psd_mean<<<dim3((NBIN + 255) / 256, (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), 256, 0, st>>>(
+        k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), PSD_T, 0, st>>>(
             P, n_seg, (int)seg_step, (int)K, psd, n_psd);
     }
     AFG_LAUNCH_CHECK(ctx, "k_psd_mean");
@@ -794,7 +837,7 @@ int launch_psd_rows(afg_ctx *ctx, const float *const *rows_dev, int n_rows, int6
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
         KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_rows * (K * 4.0 + 8.0) * NBIN);
-        k_psd_mean<<<dim3((NBIN + 255) / 256, 1, (unsigned)n_rows), 256, 0, st>>>(P, K, 0, (int)K, psd, 1);
+        k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), 1, (unsigned)n_rows), PSD_T, 0, st>>>(P, K, 0, (int)K, psd, 1);
     }
     AFG_LAUNCH_CHECK(ctx, "k_psd_mean");
     return AFG_OK;
@@ -839,7 +882,7 @@ cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, i
                                                                              psd_scale(K, fs));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_psd_mean<<<dim3((NBIN + 255) / 256, (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), 256, 0, st>>>(
+    k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), PSD_T, 0, st>>>(
         P, n_seg, (int)seg_step, (int)K, psd, n_psd);
     return cudaGetLastError();
 }
