@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(T32_T, 1) k_tiny32(const T32Args a) {
         sm.x[s] = 0.f;
         sm.h[s] = 0.f;
     }
+    cluster_sync_all();  // both CTAs have started: their shared memory may be written
     for (; win < a.n_win; win += n_clusters, buf ^= 1) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
