@@ -5,12 +5,12 @@
 //   taps       h_m = (1/N) sum_k A_k e^{+2 pi i k m / N},  g_m = sqrt(2/fs) taper(m) h_m,  |m| <= F/2
 //   gains      G_k = sum_m g_m e^{-2 pi i k m / N}, real (g is even), stored as FP32 divided by NC
 //
-// k_filter (F <= 2048): the whole build of one or two filters in one CTA, in pairs of floats (high + low
+// k_filter_pair, k_filter_one (F <= 2048): the whole build on chip, in pairs of floats (high + low
 // part, about 46 bits; the sums and products are the error-free transformations of Dekker and Knuth).  The
 // gains are FP32, so the pairs' error is 2^-20 of their rounding.  This GPU retires 2 FP64 FMAs a clock and SM
 // against 128 FP32 ones, and a pair operation takes 8 FP32 instructions: three FP64 kernels with their
 // intermediate transforms in memory took 5.0 ms for 5402 filters (FP64 pipe 85 % busy) and 41 us for two; this
-// takes 0.95 ms and 30 us, and the whitened strain differs by 7e-10 of its norm (its error is 1.2e-6).
+// takes 0.95 ms and 22 us, and the whitened strain differs by 7e-10 of its norm (its error is 1.2e-6).
 // k_filter_build (longer filters): one CTA per filter, FP64.
 #include <math.h>
 
@@ -100,10 +100,12 @@ __device__ __forceinline__ dc norm(dc a) {
     const float2 s = add2(a.h, a.l);
     return {s, sub2(a.l, sub2(s, a.h))};
 }
-template <int S>
-__device__ __forceinline__ dc mul_i(dc a) {  // a S i
-    return S < 0 ? dc{make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x)}
-                 : dc{make_float2(-a.h.y, a.h.x), make_float2(-a.l.y, a.l.x)};
+__device__ __forceinline__ dc mul_ni(dc a) { return {make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x)}; }  // -i a
+// both parts times a real pair (c + cl): product, its error and the cross terms
+__device__ __forceinline__ dc scale(dc a, float c, float cl) {
+    const float2 C = make_float2(c, c), p = __fmul2_rn(a.h, C);
+    const float2 e = __ffma2_rn(a.h, C, make_float2(-p.x, -p.y));
+    return {p, __ffma2_rn(a.l, C, __ffma2_rn(a.h, make_float2(cl, cl), e))};
 }
 __device__ __forceinline__ dd add(dd a, dd b) {
     const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
@@ -118,20 +120,26 @@ __device__ __forceinline__ dd neg(dd a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ dd re(dc a) { return {a.h.x, a.l.x}; }
 __device__ __forceinline__ dd im(dc a) { return {a.h.y, a.l.y}; }
 __device__ __forceinline__ dc cmk(dd a, dd b) { return {make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
-// a w, or a conj(w) for CONJ
-template <bool CONJ>
+// a w = (a.re, a.re) (w.re, w.im) + (a.im, a.im) (-w.im, w.re), both products and their sum packed
 __device__ __forceinline__ dc cmul(dc a, dc w) {
-    const dd ar = re(a), ai = im(a), wr = re(w), wi = CONJ ? neg(im(w)) : im(w);
-    return cmk(add(mul(ar, wr), neg(mul(ai, wi))), add(mul(ar, wi), mul(ai, wr)));
+    const float2 A = make_float2(a.h.x, a.h.x), B = make_float2(a.h.y, a.h.y);
+    const float2 Al = make_float2(a.l.x, a.l.x), Bl = make_float2(a.l.y, a.l.y);
+    const float2 V = make_float2(-w.h.y, w.h.x), Vl = make_float2(-w.l.y, w.l.x);
+    const float2 p = __fmul2_rn(A, w.h), q = __fmul2_rn(B, V);
+    float2 e = __ffma2_rn(A, w.h, make_float2(-p.x, -p.y));
+    e = __ffma2_rn(Al, w.h, __ffma2_rn(A, w.l, e));
+    float2 f = __ffma2_rn(B, V, make_float2(-q.x, -q.y));
+    f = __ffma2_rn(Bl, V, __ffma2_rn(B, Vl, f));
+    return cadd(dc{p, e}, dc{q, f});
 }
 __device__ __forceinline__ float4 pk(dc a) { return make_float4(a.h.x, a.h.y, a.l.x, a.l.y); }
 __device__ __forceinline__ dc up(float4 v) { return {make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
 __host__ __device__ constexpr float hi_of(double v) { return (float)v; }
 __host__ __device__ constexpr float lo_of(double v) { return (float)(v - (double)(float)v); }
 
-template <int S>
+// DFTs with the kernel e^{-2 pi i / n}
 __device__ __forceinline__ void dft4(dc &a, dc &b, dc &c, dc &d) {
-    const dc e0 = cadd(a, c), e1 = csub(a, c), o0 = cadd(b, d), o1 = mul_i<S>(csub(b, d));
+    const dc e0 = cadd(a, c), e1 = csub(a, c), o0 = cadd(b, d), o1 = mul_ni(csub(b, d));
     a = cadd(e0, o0);
     c = csub(e0, o0);
     b = cadd(e1, o1);
@@ -140,37 +148,36 @@ __device__ __forceinline__ void dft4(dc &a, dc &b, dc &c, dc &d) {
 constexpr double R_HALF = 0.70710678118654752440084436210485;  // cos(pi / 4)
 constexpr double C_PI8 = 0.92387953251128675612818318939679;   // cos(pi / 8)
 constexpr double S_PI8 = 0.38268343236508977172845998403040;   // sin(pi / 8)
-// a e^{S i pi q / 8}, q = 1, 2, 3, 6, 9 (the turns a radix-16 or radix-8 butterfly needs)
-template <int S, int Q>
+// a e^{-i pi q / 8}, q = 1, 2, 3, 6, 9 (the turns a radix-16 or radix-8 butterfly needs)
+template <int Q>
 __device__ __forceinline__ dc turn(dc a) {
-    constexpr double c = Q == 1 ? C_PI8 : Q == 2 ? R_HALF : Q == 3 ? S_PI8 : Q == 6 ? -R_HALF : -C_PI8;
-    constexpr double s = Q == 1 ? S_PI8 : Q == 2 ? R_HALF : Q == 3 ? C_PI8 : Q == 6 ? R_HALF : -S_PI8;
-    const dc w = {make_float2(hi_of(c), S * hi_of(s)), make_float2(lo_of(c), S * lo_of(s))};
-    return cmul<false>(a, w);
+    if (Q == 2) return scale(cadd(a, mul_ni(a)), hi_of(R_HALF), lo_of(R_HALF));
+    if (Q == 6) return scale(csub(mul_ni(a), a), hi_of(R_HALF), lo_of(R_HALF));
+    constexpr double c = Q == 1 ? C_PI8 : Q == 3 ? S_PI8 : -C_PI8;
+    constexpr double s = Q == 1 ? S_PI8 : Q == 3 ? C_PI8 : -S_PI8;
+    return cmul(a, dc{make_float2(hi_of(c), -hi_of(s)), make_float2(lo_of(c), -lo_of(s))});
 }
 // 16-point DFT as 4 x 4; output m = k1 + 4 k2 is left in v[4 k1 + k2]
-template <int S>
 __device__ __forceinline__ void dft16(dc (&v)[16]) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) dft4<S>(v[c], v[c + 4], v[c + 8], v[c + 12]);
-    v[5] = turn<S, 1>(v[5]);
-    v[6] = turn<S, 2>(v[6]);
-    v[7] = turn<S, 3>(v[7]);
-    v[9] = turn<S, 2>(v[9]);
-    v[10] = mul_i<S>(v[10]);
-    v[11] = turn<S, 6>(v[11]);
-    v[13] = turn<S, 3>(v[13]);
-    v[14] = turn<S, 6>(v[14]);
-    v[15] = turn<S, 9>(v[15]);
+    for (int c = 0; c < 4; ++c) dft4(v[c], v[c + 4], v[c + 8], v[c + 12]);
+    v[5] = turn<1>(v[5]);
+    v[6] = turn<2>(v[6]);
+    v[7] = turn<3>(v[7]);
+    v[9] = turn<2>(v[9]);
+    v[10] = mul_ni(v[10]);
+    v[11] = turn<6>(v[11]);
+    v[13] = turn<3>(v[13]);
+    v[14] = turn<6>(v[14]);
+    v[15] = turn<9>(v[15]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dft4<S>(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    for (int k = 0; k < 4; ++k) dft4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
 }
 // 8-point DFT of v[0..8) in natural order
-template <int S>
 __device__ __forceinline__ void dft8(dc *v) {
-    dft4<S>(v[0], v[2], v[4], v[6]);
-    dft4<S>(v[1], v[3], v[5], v[7]);
-    const dc o0 = v[1], o1 = turn<S, 2>(v[3]), o2 = mul_i<S>(v[5]), o3 = turn<S, 6>(v[7]);
+    dft4(v[0], v[2], v[4], v[6]);
+    dft4(v[1], v[3], v[5], v[7]);
+    const dc o0 = v[1], o1 = turn<2>(v[3]), o2 = mul_ni(v[5]), o3 = turn<6>(v[7]);
     const dc e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
     v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
     v[1] = cadd(e1, o1); v[5] = csub(e1, o1);
@@ -227,10 +234,9 @@ __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, %
 
 // 2048-point transform of a group of 128 threads: in, v[r] = x[t + 128 r]; out, v[8 q + r] = X[t + 128 q + 256 r].
 // Radix 16, 16, 8 (Stockham); one pad slot in 17 makes every 16-byte access conflict-free.
-template <int S>
 __device__ __forceinline__ void fft2048(dc (&v)[16], float4 *d, int t, int g) {
     auto tw = [&](int i) { return up(__ldg(&g_ftab[i])); };
-    dft16<S>(v);
+    dft16(v);
 #pragma unroll
     for (int m = 0; m < 16; ++m) d[fpad(t * 16 + m)] = pk(norm(v[4 * (m & 3) + (m >> 2)]));
     group_sync(g);
@@ -238,8 +244,8 @@ __device__ __forceinline__ void fft2048(dc (&v)[16], float4 *d, int t, int g) {
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = up(d[fpad(t + FGT * r)]);
 #pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = cmul<(S > 0)>(v[r], tw(8 * r * k));
-    dft16<S>(v);
+    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], tw(8 * r * k));
+    dft16(v);
     group_sync(g);
 #pragma unroll
     for (int m = 0; m < 16; ++m) d[fpad((t - k) * 16 + k + 16 * m)] = pk(norm(v[4 * (m & 3) + (m >> 2)]));
@@ -250,8 +256,8 @@ __device__ __forceinline__ void fft2048(dc (&v)[16], float4 *d, int t, int g) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) v[8 * q + r] = up(d[fpad(j + 256 * r)]);
 #pragma unroll
-        for (int r = 1; r < 8; ++r) v[8 * q + r] = cmul<(S > 0)>(v[8 * q + r], tw(r * j));
-        dft8<S>(v + 8 * q);
+        for (int r = 1; r < 8; ++r) v[8 * q + r] = cmul(v[8 * q + r], tw(r * j));
+        dft8(v + 8 * q);
     }
 }
 
@@ -297,89 +303,105 @@ __device__ __forceinline__ dd amplitude(long long b, int s) {
 // g (w_r1 + i w_r2) is G_{8 j + r1} + i G_{8 j + r2}.  The pairs are (0, 4) and (1, 2) of a filter, and residue 3 of two
 // filters (f: the real and the imaginary part of C conj(w_3)).
 //
-// One CTA builds NF filters with 2 NF + 1 transforms side by side, 128 threads each; amplitudes, taps and gains
-// stay in shared memory, so a filter costs one read of its PSD and one write of its gains.  Amplitudes are scaled by the power of two that brings the largest near 1 (strain PSDs are near
-// 1e-46), undone in the gains.  NF = 2 shares residue 3 (5 transforms for two filters instead of 6).
-// Bound by the FP32 pipe.
-template <int NF>
-struct FilterGeo {
-    static constexpr int NG = 2 * NF + 1, T = NG * FGT;
-    static constexpr int ARS = 1026, GRS = 1028;  // rows of the amplitudes (float2) and gains by residue: no conflicts
-    static constexpr int REGION = NG * FSLOTS * 16;
-    static constexpr int AMP = NF * FP * ARS * 8;
-    static constexpr int TAPS = REGION > AMP ? REGION : AMP;  // the taps follow, never overlaid
-    static constexpr int BYTES = TAPS + NF * 1024 * 8;
+// The inverse transform is conj(FFT(conj x)): the second residue enters negated and the result is read as its
+// conjugate.  Amplitudes are scaled by the power of two that brings the largest near 1 (strain PSDs are near 1e-46),
+// undone in the gains.
+constexpr int ARS = 1026, GRS = 1028;  // rows of the amplitudes (float2) and gains by residue: no bank conflicts
+
+// bits of a PSD value that has an amplitude, else 0 (below the highpass; infinity: amplitude 0; NaN; not positive)
+__device__ __forceinline__ long long psd_bits(long long b, int k, int k_hp) {
+    return k < k_hp || b >= 0x7FF0000000000000LL || b < 0 ? 0LL : b;
+}
+// the gains' scale 2^-s in two exact steps (past the floats' range: 0 or infinity, as the FP64 gain would round)
+struct Unscale {
+    float p1, p2;
+    __device__ __forceinline__ Unscale(int emin) {
+        const int s = emin < (1 << 20) ? (emin - 1023) >> 1 : 0;
+        const int e1 = max(-126, min(127, -s)), e2 = max(-126, min(127, -s - e1));
+        p1 = __int_as_float((127 + e1) << 23);
+        p2 = __int_as_float((127 + e2) << 23);
+    }
+    __device__ __forceinline__ float operator()(float g) const { return g * p1 * p2; }
 };
 
-template <int NF>
-__global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__restrict__ psd, int64_t nf, int k_hp,
-                                                                const float2 *__restrict__ tap,
-                                                                float *__restrict__ gains) {
-    using Geo = FilterGeo<NF>;
+// f(n) of conj C and the turn w: Re(C conj w) and Im(C conj w)
+__device__ __forceinline__ dd f_re(dc c, dc w) { return add(mul(re(c), re(w)), neg(mul(im(c), im(w)))); }
+__device__ __forceinline__ dd f_im(dc c, dc w) { return neg(add(mul(im(c), re(w)), mul(re(c), im(w)))); }
+
+// Many filters: one CTA builds two with five transforms side by side, 128 threads each; amplitudes, taps and gains
+// stay in shared memory, so a filter costs one read of its PSD and one write of its gains.
+// Bound by the instructions of the pair arithmetic (20 warps of 96 registers, 48 % of the issue slots).
+constexpr int F2_NG = 5, F2_T = F2_NG * FGT;
+constexpr int F2_REGION = F2_NG * FSLOTS * 16;  // amplitudes, transforms and gains, one after the other; then the taps
+constexpr int F2_BYTES = F2_REGION + 2 * 1024 * 8;
+static_assert(2 * FP * ARS * 8 <= F2_REGION && 2 * FP * GRS * 4 <= F2_REGION, "overlaid stages");
+
+__global__ void __launch_bounds__(F2_T, 1) k_filter_pair(const double *__restrict__ psd, int64_t nf, int k_hp,
+                                                         const float2 *__restrict__ tap, float *__restrict__ gains) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int emin[NF];
-    float2 *amp = reinterpret_cast<float2 *>(smem_raw);  // [NF][FP][ARS]: A_{8 i + rho}
-    float2 *taps = reinterpret_cast<float2 *>(smem_raw + Geo::TAPS);
-    float *gst = reinterpret_cast<float *>(smem_raw);    // [NF][FP][GRS]
+    __shared__ int emin[2];
+    float2 *amp = reinterpret_cast<float2 *>(smem_raw);  // [2][FP][ARS]: A_{8 i + rho}
+    float2 *taps = reinterpret_cast<float2 *>(smem_raw + F2_REGION);
+    float *gst = reinterpret_cast<float *>(smem_raw);    // [2][FP][GRS]
     const int tid = threadIdx.x, g = tid / FGT, t = tid % FGT;
-    const int64_t f0 = (int64_t)blockIdx.x * NF;
-    const int n_here = (int)min((int64_t)NF, nf - f0);
+    const int64_t f0 = (int64_t)blockIdx.x * 2;
+    const int n_here = (int)min((int64_t)2, nf - f0);
     float4 *d = reinterpret_cast<float4 *>(smem_raw) + g * FSLOTS;
 
     // ---- amplitudes: every PSD value is loaded once, all loads in flight together
-    constexpr int PER = (NF * NBIN + Geo::T - 1) / Geo::T;
-    if (tid < NF) emin[tid] = 1 << 20;
-    long long b[PER];
+    {
+        constexpr int PER = (2 * NBIN + F2_T - 1) / F2_T;
+        if (tid < 2) emin[tid] = 1 << 20;
+        long long b[PER];
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int x = tid + i * Geo::T, k = NF == 1 || x < NBIN ? x : x - NBIN;
-        b[i] = x < n_here * NBIN ? __ldg(reinterpret_cast<const long long *>(psd) + f0 * NBIN + x) : 0LL;
-        if (k < k_hp || b[i] >= 0x7FF0000000000000LL) b[i] = 0LL;  // (infinity: amplitude 0; NaN; negative stays < 0)
-    }
-    __syncthreads();
-    int e[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) e[f] = 1 << 20;
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-        if (b[i] > 0) {
-            const int x = exp_of(b[i]), f = NF == 1 || tid + i * Geo::T < NBIN ? 0 : NF - 1;
-            if (f == 0) e[0] = min(e[0], x);
-            else e[NF - 1] = min(e[NF - 1], x);
+        for (int i = 0; i < PER; ++i) {
+            const int x = tid + i * F2_T;
+            b[i] = x < n_here * NBIN ? __ldg(reinterpret_cast<const long long *>(psd) + f0 * NBIN + x) : 0LL;
+            b[i] = psd_bits(b[i], x < NBIN ? x : x - NBIN, k_hp);
         }
+        __syncthreads();
+        int e0 = 1 << 20, e1 = 1 << 20;
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        e[f] = __reduce_min_sync(0xffffffffu, e[f]);
-        if ((tid & 31) == 0) atomicMin(&emin[f], e[f]);
-    }
-    __syncthreads();
+        for (int i = 0; i < PER; ++i)
+            if (b[i]) {
+                const int x = exp_of(b[i]);
+                if (tid + i * F2_T < NBIN) e0 = min(e0, x);
+                else e1 = min(e1, x);
+            }
+        e0 = __reduce_min_sync(0xffffffffu, e0);
+        e1 = __reduce_min_sync(0xffffffffu, e1);
+        if ((tid & 31) == 0) {
+            atomicMin(&emin[0], e0);
+            atomicMin(&emin[1], e1);
+        }
+        __syncthreads();
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int x = tid + i * Geo::T, f = NF == 1 || x < NBIN ? 0 : NF - 1, k = x - f * NBIN;
-        if (x >= NF * NBIN) break;
-        dd a = {0.f, 0.f};
-        if (b[i] > 0) a = amplitude(b[i], (emin[f] - 1023) >> 1);
-        amp[(f * FP + (k & 7)) * Geo::ARS + (k >> 3)] = make_float2(a.h, a.l);
+        for (int i = 0; i < PER; ++i) {
+            const int x = tid + i * F2_T, f = x < NBIN ? 0 : 1, k = x - f * NBIN;
+            if (x >= 2 * NBIN) break;
+            dd a = {0.f, 0.f};
+            if (b[i]) a = amplitude(b[i], (emin[f] - 1023) >> 1);
+            amp[(f * FP + (k & 7)) * ARS + (k >> 3)] = make_float2(a.h, a.l);
+        }
+        __syncthreads();
     }
-    __syncthreads();
 
     // ---- inverse transforms: this group's kind (0: residues 0 and 4, 1: 1 and 2, 2: 3 of both filters) and filter
-    const int kind = g == 2 * NF ? 2 : g & 1, fa = g == 2 * NF ? 0 : g >> 1;
+    const int kind = g == 4 ? 2 : g & 1, fa = g == 4 ? 0 : g >> 1;
     const int r1 = kind == 0 ? 0 : kind == 1 ? 1 : 3, r2 = kind == 0 ? 4 : kind == 1 ? 2 : 3;
     auto amp_at = [&](int f, int r, int j) {  // A_{8 j + r}, j in [0, 2048): bins past N/2 are mirrored
-        if (j < 1024) return amp[(f * FP + r) * Geo::ARS + j];
-        return r == 0 ? amp[f * FP * Geo::ARS + 2048 - j] : amp[(f * FP + 8 - r) * Geo::ARS + 2047 - j];
+        if (j < 1024) return amp[(f * FP + r) * ARS + j];
+        return r == 0 ? amp[f * FP * ARS + 2048 - j] : amp[(f * FP + 8 - r) * ARS + 2047 - j];
     };
     dc v[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
         const int j = t + FGT * r;
-        const float2 a = amp_at(fa, r1, j);
-        const float2 b = kind < 2 ? amp_at(fa, r2, j) : NF == 2 ? amp_at(NF - 1, 3, j) : make_float2(0.f, 0.f);
-        v[r] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+        const float2 a = amp_at(fa, r1, j), b = amp_at(kind < 2 ? fa : 1, r2, j);
+        v[r] = {make_float2(a.x, -b.x), make_float2(a.y, -b.y)};
     }
     __syncthreads();  // the amplitudes are read: the transforms overwrite them
-    fft2048<+1>(v, d, t, g);
+    fft2048(v, d, t, g);
     group_sync(g);
     const float4 *wt = g_ftab + (1 + kind) * FL;
     float2 *fs = reinterpret_cast<float2 *>(d);  // f(n) [2048], and of the second filter behind it
@@ -389,21 +411,21 @@ __global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__
         for (int r = 0; r < 8; ++r) {
             const int n = t + FGT * q + 256 * r;
             const dc c = v[8 * q + r], w = up(__ldg(&wt[n]));
-            const dd a = add(mul(re(c), re(w)), mul(im(c), im(w)));
+            const dd a = f_re(c, w);
             fs[n] = make_float2(a.h, a.l);
             if (kind == 2) {
-                const dd b = add(mul(im(c), re(w)), neg(mul(re(c), im(w))));
+                const dd b = f_im(c, w);
                 fs[FL + n] = make_float2(b.h, b.l);
             }
         }
     __syncthreads();
 
     // ---- taps g_m, m in [0, 1024)
-    for (int i = tid; i < NF * 1024; i += Geo::T) {
+    for (int i = tid; i < 2 * 1024; i += F2_T) {
         const int f = i >> 10, m = i & 1023, mm = (FL - m) & (FL - 1);
         const float2 *s04 = reinterpret_cast<const float2 *>(smem_raw + (size_t)(2 * f) * FSLOTS * 16);
         const float2 *s12 = reinterpret_cast<const float2 *>(smem_raw + (size_t)(2 * f + 1) * FSLOTS * 16);
-        const float2 *s3 = reinterpret_cast<const float2 *>(smem_raw + (size_t)(2 * NF) * FSLOTS * 16) + f * FL;
+        const float2 *s3 = reinterpret_cast<const float2 *>(smem_raw + (size_t)4 * FSLOTS * 16) + f * FL;
         auto pair = [&](const float2 *s) { return add(dd{s[m].x, s[m].y}, dd{s[mm].x, s[mm].y}); };
         const dd z = pair(s04);
         const float2 tp = __ldg(&tap[m]);
@@ -422,14 +444,9 @@ __global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__
             return dd{a.x, a.y};
         };
         const dd a = tp(fa);
-        if (NF == 2 && kind == 2) {  // (g_a + i g_b) w_3
-            const dd b = tp(NF - 1);
-            v[r] = cmul<false>(cmk(a, b), w);
-        } else {
-            v[r] = cmk(mul(a, re(w)), mul(a, im(w)));
-        }
+        v[r] = kind == 2 ? cmul(cmk(a, tp(1)), w) : cmk(mul(a, re(w)), mul(a, im(w)));  // (g_a + i g_b) w_3
     }
-    fft2048<-1>(v, d, t, g);
+    fft2048(v, d, t, g);
     __syncthreads();  // every transform has left shared memory: the gains overlay it
     auto put = [&](int f, int r, int j, float x) {
         int k = 8 * j + r;
@@ -437,7 +454,7 @@ __global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__
             if (r == 0 || r == 4) return;  // its own mirror
             k = NFFT - k;
         }
-        gst[(f * FP + (k & 7)) * Geo::GRS + (k >> 3)] = x;
+        gst[(f * FP + (k & 7)) * GRS + (k >> 3)] = x;
     };
 #pragma unroll
     for (int q = 0; q < 2; ++q)
@@ -446,18 +463,152 @@ __global__ void __launch_bounds__(FilterGeo<NF>::T, 1) k_filter(const double *__
             const int j = t + FGT * q + 256 * r;
             const dc c = v[8 * q + r];
             put(fa, r1, j, __fadd_rn(c.h.x, c.l.x));
-            if (kind < 2) put(fa, r2, j, __fadd_rn(c.h.y, c.l.y));
-            else if (NF == 2) put(NF - 1, 3, j, __fadd_rn(c.h.y, c.l.y));
+            put(kind < 2 ? fa : 1, r2, j, __fadd_rn(c.h.y, c.l.y));
         }
     __syncthreads();
     for (int f = 0; f < n_here; ++f) {
-        // undo the scale 2^s in two exact steps (past the floats' range: 0 or infinity, as the FP64 gain would round)
-        const int s = emin[f] < (1 << 20) ? (emin[f] - 1023) >> 1 : 0;
-        const int e1 = max(-126, min(127, -s)), e2 = max(-126, min(127, -s - e1));
-        const float p1 = __int_as_float((127 + e1) << 23), p2 = __int_as_float((127 + e2) << 23);
+        const Unscale un(emin[f]);
         float *out = gains + (f0 + f) * NBIN;
-        for (int k = tid; k < NBIN; k += Geo::T) out[k] = gst[(f * FP + (k & 7)) * Geo::GRS + (k >> 3)] * p1 * p2;
+        for (int k = tid; k < NBIN; k += F2_T) out[k] = un(gst[(f * FP + (k & 7)) * GRS + (k >> 3)]);
     }
+}
+
+// Few filters (an epoch refresh, one span): one filter per cluster of three CTAs, a transform each, so that one
+// filter's chain of pair operations runs on three SMs (two filters: about 31 us as one CTA of 384 threads each,
+// 22 us now).  Each CTA scans the whole PSD for the scale, forms the amplitudes of its own residues, and sends its
+// part of the taps to the other two through distributed shared memory.
+constexpr int F1_REGION = FSLOTS * 16;
+constexpr int F1_BYTES = F1_REGION + 4 * 1024 * 8;  // then the three parts of the taps, and the taps
+static_assert(4 * ARS * 8 <= F1_REGION, "overlaid stages");
+
+__device__ __forceinline__ void st_cluster(float2 *local, int rank, float2 v) {  // the same variable of CTA `rank`
+    uint32_t p;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+
+__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(FGT) k_filter_one(const double *__restrict__ psd, int k_hp,
+                                                                             const float2 *__restrict__ tap,
+                                                                             float *__restrict__ gains) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int emin;
+    float2 *amp = reinterpret_cast<float2 *>(smem_raw);  // rows of the residues (r1, 8 - r1, r2, 8 - r2), or (r1, r2)
+    float2 *parts = reinterpret_cast<float2 *>(smem_raw + F1_REGION), *taps = parts + 3 * 1024;
+    float4 *d = reinterpret_cast<float4 *>(smem_raw);
+    const int t = threadIdx.x, kind = blockIdx.x % 3;
+    const int64_t f = blockIdx.x / 3;
+    const long long *p = reinterpret_cast<const long long *>(psd) + f * NBIN;
+    const int r1 = kind == 0 ? 0 : kind == 1 ? 1 : 3, r2 = kind == 0 ? 4 : kind == 1 ? 2 : -1;
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");  // (waited for before the first remote store)
+    if (t == 0) emin = 1 << 20;
+    __syncthreads();
+    constexpr int BATCH = 33;  // 2 x 33 x 128 >= NBIN
+    int e = 1 << 20;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        long long b[BATCH];
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) {
+            const int k = t + FGT * (BATCH * h + i);
+            b[i] = k < NBIN ? psd_bits(__ldg(p + k), k, k_hp) : 0LL;
+        }
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i)
+            if (b[i]) e = min(e, exp_of(b[i]));
+    }
+    e = __reduce_min_sync(0xffffffffu, e);
+    if ((t & 31) == 0) atomicMin(&emin, e);
+    __syncthreads();
+    // amplitudes A_{8 i + rho} of this CTA's residues: row 0 rho = r1, 1: 8 - r1, 2: r2, 3: 8 - r2 (kind 0: 0 and 4 are
+    // their own mirrors, rows 0 and 2)
+    const int s = (emin - 1023) >> 1;
+    for (int row = 0; row < (r2 < 0 ? 2 : 4); ++row) {
+        if (kind == 0 && (row & 1)) continue;
+        const int rho = row == 0 ? r1 : row == 1 ? 8 - r1 : row == 2 ? r2 : 8 - r2;
+#pragma unroll 8
+        for (int i = t; i < 1024 + (rho == 0); i += FGT) {
+            const int k = 8 * i + rho;
+            const long long b = psd_bits(__ldg(p + k), k, k_hp);
+            dd a = {0.f, 0.f};
+            if (b) a = amplitude(b, s);
+            amp[row * ARS + i] = make_float2(a.h, a.l);
+        }
+    }
+    __syncthreads();
+    auto amp_at = [&](int row, int r, int j) {  // A_{8 j + r}, j in [0, 2048): bins past N/2 are mirrored
+        if (j < 1024) return amp[row * ARS + j];
+        return r == 0 ? amp[row * ARS + 2048 - j] : amp[(row + (kind != 0)) * ARS + 2047 - j];
+    };
+    const float4 *wt = g_ftab + (1 + kind) * FL;
+    dc v[16];
+    // the transform's code exists once, in a loop over the two stages
+#pragma unroll 1
+    for (int stage = 0; stage < 2; ++stage) {
+        if (stage == 0) {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int j = t + FGT * r;
+                const float2 a = amp_at(0, r1, j), b = r2 < 0 ? make_float2(0.f, 0.f) : amp_at(2, r2, j);
+                v[r] = {make_float2(a.x, -b.x), make_float2(a.y, -b.y)};
+            }
+            __syncthreads();  // the amplitudes are read: the transform overwrites them
+        } else {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int n = t + FGT * r, m = n <= 1024 ? n : FL - n;
+                const dc w = up(__ldg(&wt[n]));
+                const float2 a = m < 1024 ? taps[m] : make_float2(0.f, 0.f);
+                v[r] = cmk(mul(dd{a.x, a.y}, re(w)), mul(dd{a.x, a.y}, im(w)));
+            }
+        }
+        fft2048(v, d, t, 0);
+        if (stage == 1) break;
+        __syncthreads();
+        float2 *fs = reinterpret_cast<float2 *>(d);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int n = t + FGT * q + 256 * r;
+                const dd a = f_re(v[8 * q + r], up(__ldg(&wt[n])));
+                fs[n] = make_float2(a.h, a.l);
+            }
+        __syncthreads();
+        asm volatile("barrier.cluster.wait;" ::: "memory");  // every CTA of the cluster has started
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int m = t + FGT * i, mm = (FL - m) & (FL - 1);
+            const dd z = add(dd{fs[m].x, fs[m].y}, dd{fs[mm].x, fs[mm].y});
+            const float c = kind == 0 ? 0.5f : 1.f;
+            for (int o = 0; o < 3; ++o) st_cluster(parts + kind * 1024 + m, o, make_float2(c * z.h, c * z.l));
+        }
+        asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int m = t + FGT * i;
+            auto part = [&](int o) { return dd{parts[o * 1024 + m].x, parts[o * 1024 + m].y}; };
+            const float2 tp = __ldg(&tap[m]);
+            const dd h = mul(add(add(part(0), part(1)), part(2)), dd{tp.x, tp.y});
+            taps[m] = make_float2(h.h, h.l);
+        }
+        __syncthreads();
+    }
+    const Unscale un(emin);
+    float *out = gains + f * NBIN;
+    auto put = [&](int r, int j, float x) {
+        const int k = 8 * j + r;
+        if (k <= NFFT / 2) out[k] = un(x);
+        else if (r != 0 && r != 4) out[NFFT - k] = un(x);
+    };
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int j = t + FGT * q + 256 * r;
+            const dc c = v[8 * q + r];
+            put(r1, j, __fadd_rn(c.h.x, c.l.x));
+            if (r2 >= 0) put(r2, j, __fadd_rn(c.h.y, c.l.y));
+        }
 }
 
 // Fill the tables of the current device once per process (complete when this returns).
@@ -478,9 +629,9 @@ cudaError_t ensure_filter_tables() {
     cudaStreamDestroy(st);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_filter<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FilterGeo<1>::BYTES);
+        e = cudaFuncSetAttribute(k_filter_one, cudaFuncAttributeMaxDynamicSharedMemorySize, F1_BYTES);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_filter<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, FilterGeo<2>::BYTES);
+        e = cudaFuncSetAttribute(k_filter_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, F2_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_filter_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)((NC + 1) * sizeof(double2)));
@@ -533,10 +684,10 @@ int launch_filter(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, flo
     if (ctx->cfg.fir_len <= FILTER_LAGS) {
         const int k_hp = first_bin(ctx->cfg.f_highpass, ctx->cfg.fs);
         const float2 *tap = static_cast<const float2 *>(ctx->filter_tab);
-        if (nf <= 152)  // one filter per SM: the shorter CTA; more: two filters share a transform
-            k_filter<1><<<(unsigned)nf, FilterGeo<1>::T, FilterGeo<1>::BYTES, st>>>(psd, nf, k_hp, tap, gains);
+        if (nf <= 152)  // fewer pairs than half of the SMs: three CTAs a filter
+            k_filter_one<<<(unsigned)(3 * nf), FGT, F1_BYTES, st>>>(psd, k_hp, tap, gains);
         else
-            k_filter<2><<<(unsigned)((nf + 1) / 2), FilterGeo<2>::T, FilterGeo<2>::BYTES, st>>>(psd, nf, k_hp, tap, gains);
+            k_filter_pair<<<(unsigned)((nf + 1) / 2), F2_T, F2_BYTES, st>>>(psd, nf, k_hp, tap, gains);
     } else {
         k_filter_build<<<dim3((unsigned)n_psd, n_det), NT64, (NC + 1) * sizeof(double2), st>>>(
             psd, n_psd, (double)ctx->cfg.fs, ctx->cfg.f_highpass, ctx->cfg.fir_len,
