@@ -313,12 +313,16 @@ __device__ __forceinline__ int64_t plane_row(const Planes &o, int64_t w, int r) 
 // units (at most GN_U) in registers and reads raw once; else each pass reads it again.  The mean and
 // the centred variance are two passes in a fixed order, as in k_groupnorm_st.
 // Bound by memory: 4 B read + 6 B written (+ 6 B residual) per element.  Groups are independent, so a
-// window is split over several CTAs; two fit an SM and hide each other's loads.
-constexpr int GNS_T = 256;
-constexpr int GNS_U = 6;
+// window is split over several CTAs; two fit an SM and hide each other's loads.  The residual's rows are fetched into L2
+// while the statistics are formed.
+// (Per sequence of 960 ResNet34 windows, 35 launches, 21 GB: 256 threads of 6 units at three CTAs an SM 5.51 ms, at
+// two 5.04; 512 of 3 at two CTAs 4.25, with the residual fetched into L2 before the statistics 4.06, 76 % of the
+// copy rate; 1024 of 3 4.91, 512 of 2 5.21.)
+constexpr int GNS_T = 512;
+constexpr int GNS_U = 3;
 
 template <int GS, bool REG>
-__global__ void __launch_bounds__(GNS_T, REG ? 3 : 2) k_gn_split(const float *__restrict__ raw, int64_t hs, int hr, int L,
+__global__ void __launch_bounds__(GNS_T, 2) k_gn_split(const float *__restrict__ raw, int64_t hs, int hr, int L,
                                                                  int cp, int lcg, const float *__restrict__ gamma,
                                                                  const float *__restrict__ beta, float eps,
                                                                  const Planes res, int relu, const Planes out) {
@@ -392,6 +396,16 @@ __global__ void __launch_bounds__(GNS_T, REG ? 3 : 2) k_gn_split(const float *__
         __syncthreads();
     };
     if (REG) units([&](int i, int, int ch, int t) { load(i, ch, t); });
+    static_assert(GNS_T >= 512, "one channel of an item a thread");
+    const float gm = tid < cp ? __ldg(gamma + c0 + tid) : 0.f, bt = tid < cp ? __ldg(beta + c0 + tid) : 0.f;
+    if (REG && res.p) units([&](int, int, int ch, int t) {
+        if (t < L) {
+            const __nv_bfloat16 *rp = res.p + (int64_t)(c0 / 8 + ch) * res.cs + plane_row(res, w, t + 1);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + res.ps));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + 2 * res.ps));
+        }
+    });
     reduce([](float x, int) { return x; }, [&](int q, float s) { gmean[q] = s * inv; });
     reduce(
         [&](float x, int q) {
@@ -399,10 +413,10 @@ __global__ void __launch_bounds__(GNS_T, REG ? 3 : 2) k_gn_split(const float *__
             return d * d;
         },
         [&](int q, float s) { grstd[q] = rsqrtf(s * inv + eps); });
-    for (int c = tid; c < cp; c += GNS_T) {
-        const float sc = grstd[c / GS] * gamma[c0 + c];
-        scl[c] = sc;
-        shf[c] = beta[c0 + c] - gmean[c / GS] * sc;
+    if (tid < cp) {
+        const float sc = grstd[tid / GS] * gm;
+        scl[tid] = sc;
+        shf[tid] = bt - gmean[tid / GS] * sc;
     }
     __syncthreads();
 
@@ -456,23 +470,29 @@ __global__ void __launch_bounds__(GNS_T, REG ? 3 : 2) k_gn_split(const float *__
 }
 
 // ---------------------------------------------------------------- stem
-// Convolution (FP32, the FMA order of k_stem), GroupNorm, ReLU and max-pool of one window, straight into
-// planes.  The samples sit in shared memory and the convolution (2 k FMAs an output) is evaluated three
-// times (mean, centred variance, output) instead of being stored: k_stem + k_groupnorm moved 2 MB a
-// window through memory.  grid (n_win), 512 threads; a warp takes four channels and 32 positions a step.
-constexpr int STS_T = 512;
+// Convolution (FP32, the FMA order of k_stem), GroupNorm, ReLU and max-pool of one window's channels, straight into
+// planes.  grid (C0 / cp, n_win), 256 threads: CTA (i, w) takes the channels [cp i, cp (i + 1)), whole groups; a warp
+// takes four channels and a run of positions, 32 a step, the samples in shared memory.  REG: the run is at most
+// STS_U steps and its outputs stay in registers, so the convolution (2 k FMAs and, for four channels, 2 k
+// shared-memory reads an output) is evaluated once; else three times (mean, centred variance, output).  Bound by the
+// shared-memory reads: 718 us for 960 ResNet34 windows evaluated three times, 393 now; k_stem + k_groupnorm moved
+// 2 MB a window through memory.
+constexpr int STS_T = 256, STS_W = STS_T / 32;
 constexpr int STS_K = 7;
+constexpr int STS_U = 24;
 
-__global__ void __launch_bounds__(STS_T) k_stem_split(const float *__restrict__ y, int64_t n_y, int64_t y_stride,
-                                                      int64_t first, int64_t stride, int64_t shift, int64_t w0,
-                                                      const float *__restrict__ wt, const float *__restrict__ gamma,
-                                                      const float *__restrict__ beta, int C0, int k, int s, int W, int L0,
-                                                      int pool, int G, float eps, const Planes out) {
-    extern __shared__ float xs[];  // [2][W + 2 pad], then per channel: sum, scale, shift
-    const int pad = k / 2, Wp = W + 2 * pad;
-    float *csum = xs + 2 * Wp, *scl = csum + C0, *shf = scl + C0;
+template <bool REG>
+__global__ void __launch_bounds__(STS_T, 1) k_stem_split(const float *__restrict__ y, int64_t n_y, int64_t y_stride,
+                                                         int64_t first, int64_t stride, int64_t shift, int64_t w0,
+                                                         const float *__restrict__ wt, const float *__restrict__ gamma,
+                                                         const float *__restrict__ beta, int cp, int k, int s, int W,
+                                                         int L0, int pool, int cg, float eps, const Planes out) {
+    extern __shared__ float xs[];  // [2][W + 2 pad], then sums [warps per quad][cp], mean or shift [cp], scale [cp]
+    const int pad = k / 2, Wp = W + 2 * pad, c0 = blockIdx.x * cp;
+    const int wq = max(1, 4 * STS_W / cp);  // warps that share a quad's positions
+    float *csum = xs + 2 * Wp, *shf = csum + wq * cp, *scl = shf + cp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t start = first + (w0 + blockIdx.x) * stride;
+    const int64_t start = first + (w0 + blockIdx.y) * stride;
     for (int t = tid; t < Wp; t += STS_T) {
         const int tt = t - pad;
         float a = 0.f, b = 0.f;
@@ -485,17 +505,19 @@ __global__ void __launch_bounds__(STS_T) k_stem_split(const float *__restrict__ 
         xs[t] = a;
         xs[Wp + t] = b;
     }
-    __syncthreads();
-    const int cg = C0 / G;
+    // the warp's first channels (local; more only where cp > 4 STS_W, never with REG) and its run of positions
+    const int cl0 = warp / wq * 4, cls = STS_W / wq * 4, part = warp % wq;
+    const int steps = (L0 + 31) / 32, per = (steps + wq - 1) / wq, s0 = part * per, s1 = min(steps, s0 + per);
     float wr[4][2][STS_K];
-    auto weights = [&](int c) {
+    auto weights = [&](int cl) {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int r = 0; r < STS_K; ++r) wr[e][i][r] = r < k ? wt[((c + e) * 2 + i) * k + r] : 0.f;
+                for (int r = 0; r < STS_K; ++r) wr[e][i][r] = r < k ? wt[((c0 + cl + e) * 2 + i) * k + r] : 0.f;
     };
+    weights(cl0);
     auto conv = [&](int t, float (&z)[4]) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) z[e] = 0.f;
@@ -509,82 +531,109 @@ __global__ void __launch_bounds__(STS_T) k_stem_split(const float *__restrict__ 
                     for (int e = 0; e < 4; ++e) z[e] = fmaf(wr[e][i][r], x, z[e]);
                 }
     };
-    // two passes: channel sums of the values, then of their squared distance to the group mean (in shf)
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int c = warp * 4; c < C0; c += STS_T / 32 * 4) {
-            weights(c);
-            float m[4], a[4] = {0.f, 0.f, 0.f, 0.f};
+    float v[REG ? STS_U : 1][4];
+    // body(i, step) over the warp's steps
+    auto run = [&](auto body) {
+        if (REG) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) m[e] = pass ? shf[c + e] : 0.f;
-            for (int t = lane; t < L0; t += 32) {
-                float z[4];
-                conv(t, z);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float d = z[e] - m[e];
-                    a[e] = pass ? fmaf(d, d, a[e]) : a[e] + d;
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) a[e] += __shfl_xor_sync(0xffffffffu, a[e], o);
-                if (lane == 0) csum[c + e] = a[e];
+            for (int i = 0; i < STS_U; ++i)
+                if (s0 + i < s1) body(i, s0 + i);
+        } else {
+            for (int st = s0; st < s1; ++st) {
+                conv(min(st * 32 + lane, L0 - 1), v[0]);
+                body(0, st);
             }
         }
+    };
+    __syncthreads();
+    if (REG) run([&](int i, int st) { conv(min(st * 32 + lane, L0 - 1), v[i]); });
+    // two passes: channel sums of the values, then of their squared distance to the group mean (in shf)
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+        for (int cl = cl0; cl < cp; cl += cls) {
+        if (!REG) weights(cl);
+        float m[4], a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) m[e] = pass ? shf[cl + e] : 0.f;
+        run([&](int i, int st) {
+            if (st * 32 + lane < L0)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float d = v[i][e] - m[e];
+                    a[e] = pass ? fmaf(d, d, a[e]) : a[e] + d;
+                }
+        });
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a[e] += __shfl_xor_sync(0xffffffffu, a[e], o);
+            if (lane == 0) csum[part * cp + cl + e] = a[e];
+        }
+        }
         __syncthreads();
-        for (int c = tid; c < C0; c += STS_T) {
+        for (int c = tid; c < cp; c += STS_T) {
             float t = 0.f;
-            for (int i = c / cg * cg; i < (c / cg + 1) * cg; ++i) t += csum[i];
+            for (int i = c / cg * cg; i < (c / cg + 1) * cg; ++i)
+                for (int q = 0; q < wq; ++q) t += csum[q * cp + i];
             t /= (float)L0 * (float)cg;
             if (pass == 0) {
                 shf[c] = t;
             } else {
-                const float sc = rsqrtf(t + eps) * gamma[c];
+                const float sc = rsqrtf(t + eps) * gamma[c0 + c];
                 scl[c] = sc;
-                shf[c] = beta[c] - shf[c] * sc;
+                shf[c] = beta[c0 + c] - shf[c] * sc;
             }
         }
         __syncthreads();
     }
     const int Lo = pool ? (L0 + 2 - 3) / 2 + 1 : L0;
-    for (int c = warp * 4; c < C0; c += STS_T / 32 * 4) {
-        weights(c);
-        float sc[4], sh[4], carry[4];
+#pragma unroll 1
+    for (int cl = cl0; cl < cp; cl += cls) {
+    if (!REG) weights(cl);
+    float sc[4], sh[4], carry[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        sc[e] = scl[cl + e];
+        sh[e] = shf[cl + e];
+        carry[e] = -INFINITY;
+    }
+    if (pool && s0 > 0) {  // the position before the run
+        conv(min(s0 * 32, L0) - 1, carry);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) carry[e] = fmaxf(fmaf(carry[e], sc[e], sh[e]), 0.f);
+    }
+    __nv_bfloat16 *oc = out.p + (int64_t)((c0 + cl) / 8) * out.cs + (cl & 4);
+    run([&](int i, int st) {
+        const int t = st * 32 + lane;
+        float z[4], m[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            sc[e] = scl[c + e];
-            sh[e] = shf[c + e];
-            carry[e] = -INFINITY;
-        }
-        __nv_bfloat16 *oc = out.p + (int64_t)(c / 8) * out.cs + (c & 4);
-        for (int t0 = 0; t0 < L0; t0 += 32) {
-            const int t = t0 + lane;
-            float z[4], m[4];
-            conv(min(t, L0 - 1), z);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                z[e] = t < L0 ? fmaxf(fmaf(z[e], sc[e], sh[e]), 0.f) : -INFINITY;
+            z[e] = t < L0 ? fmaxf(fmaf(v[i][e], sc[e], sh[e]), 0.f) : -INFINITY;
+            if (pool) {
                 float lo = __shfl_up_sync(0xffffffffu, z[e], 1);
                 const float hi = __shfl_down_sync(0xffffffffu, z[e], 1);
                 if (lane == 0) lo = carry[e];
-                m[e] = pool ? fmaxf(fmaxf(lo, z[e]), hi) : z[e];  // (stored by even lanes: hi is in the warp)
+                m[e] = fmaxf(fmaxf(lo, z[e]), hi);  // (stored by even lanes: hi is in the warp)
                 carry[e] = __shfl_sync(0xffffffffu, z[e], 31);
-            }
-            const int u = pool ? t >> 1 : t;
-            if (t < L0 && u < Lo && (!pool || !(lane & 1))) {
-                uint32_t p[3][2];
-                split3(m[0], m[1], p[0][0], p[1][0], p[2][0]);
-                split3(m[2], m[3], p[0][1], p[1][1], p[2][1]);
-                const int64_t o = plane_row(out, blockIdx.x, u + 1);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2 *>(oc + i * out.ps + o) = make_uint2(p[i][0], p[i][1]);
+            } else {
+                m[e] = z[e];
             }
         }
+        const int u = pool ? t >> 1 : t;
+        if (t < L0 && u < Lo && (!pool || !(lane & 1))) {
+            uint32_t p[3][2];
+            split3(m[0], m[1], p[0][0], p[1][0], p[2][0]);
+            split3(m[2], m[3], p[0][1], p[1][1], p[2][1]);
+            const int64_t o = plane_row(out, blockIdx.y, u + 1);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2 *>(oc + q * out.ps + o) = make_uint2(p[q][0], p[q][1]);
+        }
+    });
     }
-    for (int i = tid; i < C0 / 8 * 6; i += STS_T)
-        *reinterpret_cast<uint4 *>(out.p + ((i % 6) >> 1) * out.ps + (int64_t)(i / 6) * out.cs +
-                                   plane_row(out, blockIdx.x, (i & 1) ? Lo + 1 : 0)) = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < cp / 8 * 6; i += STS_T)
+        *reinterpret_cast<uint4 *>(out.p + ((i % 6) >> 1) * out.ps + (int64_t)(c0 / 8 + i / 6) * out.cs +
+                                   plane_row(out, blockIdx.y, (i & 1) ? Lo + 1 : 0)) = make_uint4(0, 0, 0, 0);
 }
 
 // ---------------------------------------------------------------- head
@@ -710,7 +759,8 @@ int net_split_prepare(afg_ctx *ctx) {
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_gn_split<GS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024))
     AFG_SPLIT_GN(2); AFG_SPLIT_GN(4); AFG_SPLIT_GN(8);
 #undef AFG_SPLIT_GN
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_split, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_split<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_split<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024));
     return AFG_OK;
 }
 
@@ -839,9 +889,23 @@ int launch_infer_split(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stri
         {
             KScope ks(ctx, st, KK_STEM, 2.0 * nw * S.lout * S.cout * S.cin * S.k,
                       4.0 * nw * ((double)2 * W + (double)P.l_after_stem * S.cout));
-            k_stem_split<<<nw, STS_T, (2 * (W + 2 * (S.k / 2)) + 3 * S.cout) * sizeof(float), st>>>(
-                y, n_y, y_stride, first, stride, shift, w0, S.wt, S.gamma, S.beta, S.cout, S.k, S.stride, W, S.lout,
-                P.net.stem_pool, P.net.groups, P.net.eps, A);
+            // channels per CTA: 32 (four a warp), fewer where that puts a warp's run of positions in registers, or a
+            // whole group
+            const int cg = S.cout / P.net.groups, steps = (S.lout + 31) / 32;
+            int cp = std::max(4 * STS_W, cg);
+            auto run = [&] {
+                const int wq = std::max(1, 4 * STS_W / cp);
+                return cp <= 4 * STS_W ? (steps + wq - 1) / wq : STS_U + 1;
+            };
+            while (run() > STS_U && cp > 8 && cp > cg) cp /= 2;
+            const size_t sm = (size_t)(2 * (W + 2 * (S.k / 2)) + std::max(4 * STS_W, cp) + 2 * cp) * sizeof(float);
+            const dim3 grid(S.cout / cp, nw);
+#define AFG_STEM(REG)                                                                                                    \
+    k_stem_split<REG><<<grid, STS_T, sm, st>>>(y, n_y, y_stride, first, stride, shift, w0, S.wt, S.gamma, S.beta, cp, S.k, \
+                                               S.stride, W, S.lout, P.net.stem_pool, cg, P.net.eps, A)
+            if (run() <= STS_U) AFG_STEM(true);
+            else AFG_STEM(false);
+#undef AFG_STEM
         }
         AFG_LAUNCH_CHECK(ctx, "k_stem_split");
         for (size_t b = 0; b < P.blocks.size(); ++b) {
