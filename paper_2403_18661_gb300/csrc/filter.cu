@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(NT64) k_filter_build(const double *__restrict_
                                                         float *__restrict__ gains) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2 *d = reinterpret_cast<double2 *>(smem_raw);
+    pdl_trigger();  // (launched plainly)
     const int64_t e = blockIdx.x;
     const int det = blockIdx.y;
     const double *p = psd + ((int64_t)det * n_psd + e) * NBIN;
@@ -487,7 +488,7 @@ __device__ __forceinline__ void st_cluster(float2 *local, int rank, float2 v) { 
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y) : "memory");
 }
 
-__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(FGT) k_filter_one(const double *__restrict__ psd, int k_hp,
+__global__ void __launch_bounds__(FGT) k_filter_one(const double *__restrict__ psd, int k_hp,
                                                                              const float2 *__restrict__ tap,
                                                                              float *__restrict__ gains) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -502,6 +503,8 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(FGT) k_filter_one(co
     asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");  // (waited for before the first remote store)
     if (t == 0) emin = 1 << 20;
     __syncthreads();
+    pdl_wait();     // the PSD
+    pdl_trigger();  // (not before: a dependent may rely on what came before this launch)
     constexpr int BATCH = 33;  // 2 x 33 x 128 >= NBIN
     int e = 1 << 20;
 #pragma unroll 1
@@ -685,7 +688,8 @@ int launch_filter(afg_ctx *ctx, const double *psd, int n_det, int64_t n_psd, flo
         const int k_hp = first_bin(ctx->cfg.f_highpass, ctx->cfg.fs);
         const float2 *tap = static_cast<const float2 *>(ctx->filter_tab);
         if (nf <= 152)  // fewer pairs than half of the SMs: three CTAs a filter
-            k_filter_one<<<(unsigned)(3 * nf), FGT, F1_BYTES, st>>>(psd, k_hp, tap, gains);
+            AFG_CUDA(ctx, launch_pdl_cluster(k_filter_one, dim3((unsigned)(3 * nf)), dim3(FGT), F1_BYTES, st, 3, psd, k_hp, tap,
+                                             gains));
         else
             k_filter_pair<<<(unsigned)((nf + 1) / 2), F2_T, F2_BYTES, st>>>(psd, nf, k_hp, tap, gains);
     } else {

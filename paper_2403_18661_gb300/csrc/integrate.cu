@@ -69,6 +69,8 @@ __global__ void __launch_bounds__(CL_T) k_cluster(const float *__restrict__ z, i
     const int len = CL_N + 2 * h;
     float *zl = cs, *A = cs + len + n_int, *B = A + len;
     const int64_t n_win = n_out + n_int - 1;
+    pdl_wait();  // the logits
+    pdl_trigger();
     for (int i = tid; i < len + n_int - 1; i += CL_T) {
         const int64_t j = j0 - h + i;
         zl[i] = j >= 0 && j < n_win ? z[j] : 0.f;
@@ -139,6 +141,7 @@ __global__ void __launch_bounds__(CL_T) k_cluster_write(const uint32_t *__restri
     __shared__ int64_t sum[CL_T / 32];
     const int tid = threadIdx.x, lane = tid & 31, t = blockIdx.x;
     int64_t s = 0;
+    pdl_wait();  // flags and counts
     if (!scanned) {
         for (int i = tid; i < t; i += CL_T) s += counts[i];
 #pragma unroll
@@ -272,19 +275,17 @@ int launch_integrate(afg_ctx *ctx, const float *logits, int64_t n_win, int n_int
         {
             KScope ks(ctx, st, KK_INTEGRATE, (double)n_out * n_int, (double)(n_win + n_out) * 4.0);
             const size_t sm = cluster_smem(h, n_int);
-            if (n_out <= CL_DIRECT && h <= CL_DIRECT_H)
-                k_cluster<true><<<(unsigned)tiles, CL_T, sm, st>>>(logits, n_out, n_int, h, stat, flags, counts, trig_idx,
-                                                                   trig_cap, n_trig);
-            else
-                k_cluster<false><<<(unsigned)tiles, CL_T, sm, st>>>(logits, n_out, n_int, h, stat, flags, counts, trig_idx,
-                                                                    trig_cap, n_trig);
+            AFG_CUDA(ctx, launch_pdl(n_out <= CL_DIRECT && h <= CL_DIRECT_H ? k_cluster<true> : k_cluster<false>,
+                                     dim3((unsigned)tiles), dim3(CL_T), sm, st, logits, n_out, (int)n_int, h, stat, flags,
+                                     counts, trig_idx, trig_cap, n_trig));
         }
         AFG_LAUNCH_CHECK(ctx, "k_cluster");
         if (tiles > 1) {
             KScope ks(ctx, st, KK_TRIGGERS, 0.0, (double)n_out / 8.0);
             const int scanned = tiles > CL_SUMS;
             if (scanned) k_trig_scan<<<1, 1024, 0, st>>>(counts, (int)tiles, n_trig);
-            k_cluster_write<<<(unsigned)tiles, CL_T, 0, st>>>(flags, counts, scanned, trig_idx, trig_cap, n_trig);
+            AFG_CUDA(ctx, launch_pdl(k_cluster_write, dim3((unsigned)tiles), dim3(CL_T), 0, st, (const uint32_t *)flags,
+                                     (const int *)counts, scanned, trig_idx, trig_cap, n_trig));
         }
         AFG_LAUNCH_CHECK(ctx, "k_cluster_write");
         return AFG_OK;

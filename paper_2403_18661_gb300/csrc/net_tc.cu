@@ -1678,7 +1678,8 @@ int launch_infer_bf16(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_strid
     KScope ks(ctx, st, KK_TINY_TC, flops_conv + flops_stem, (double)n_win * (2.0 * W * 4.0 + 4.0));
     const size_t psmem = pipe_smem(W, n_conv, a.k_stem).total;
     a.spin_ns = P.tiny_spin_ns;
-    cudaError_t e = launch_pipe(a, grid, psmem, st, false, P.tiny_ew, P.tiny_mw);
+    // a programmatic dependent of the whitening (or whatever is before): set-up overlaps its tail
+    cudaError_t e = launch_pipe(a, grid, psmem, st, true, P.tiny_ew, P.tiny_mw);
     if (e != cudaSuccess) return afg_cuda_fail(ctx, e, "k_tiny_pipe");
     return AFG_OK;
 }

@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *d = reinterpret_cast<float2 *>(smem_raw);
     float2 *u_nyq = d + SLOTS;  // U_NC (real)
+    pdl_trigger();  // (launched plainly: what it reads is complete)
     const int64_t g = blockIdx.x;
     const int det = blockIdx.y;
     const int t = threadIdx.x;
@@ -256,6 +257,8 @@ __global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P,
     const float *src = P + ((int64_t)blockIdx.z * n_seg + e0 * seg_step) * PER_ROW;
     double *dst = psd + ((int64_t)blockIdx.z * n_psd + e0) * NBIN + k;
     const int64_t ns = (int64_t)(n_e - 1) * seg_step + K;
+    pdl_wait();
+    pdl_trigger();
     bool pairs = K <= 16 && ns <= PSD_SEGS;
     if (pairs) {
         if (tid == 0) {
@@ -426,7 +429,9 @@ constexpr int WELCH_SMEM = (r16::SLOTS + 1) * (int)sizeof(float2) + (r16::NT / 3
 // when the caller's destination is the linear row lin (nullptr: always through out).
 // smem: r16::SLOTS float2 for the transform, then NBIN floats for the gains gk,
 // which are copied in asynchronously while the forward transform runs.
-template <typename Out>
+// EARLY: the samples are complete before the launch, the gains only after pdl_wait(), which comes after the forward
+// transform.
+template <bool EARLY = false, typename Out>
 __device__ __forceinline__ void whiten_block(unsigned char *smem, const float *__restrict__ src, int64_t avail,
                                              const float *__restrict__ gk, int F, int64_t cnt, Out out,
                                              float *__restrict__ lin = nullptr) {
@@ -434,7 +439,8 @@ __device__ __forceinline__ void whiten_block(unsigned char *smem, const float *_
     float2 *d = reinterpret_cast<float2 *>(smem);
     float *gs = reinterpret_cast<float *>(smem + SLOTS * sizeof(float2));
     const int t = threadIdx.x;
-    for (int k = t; k < NBIN; k += NT) cp_async4(gs + k, gk + k);
+    if (!EARLY)
+        for (int k = t; k < NBIN; k += NT) cp_async4(gs + k, gk + k);
     const int half = F / 2;
     // samples that reach a kept output (cnt + F - 1 <= 16384: indices within the block are ints)
     const int need = (int)cnt + F - 1;
@@ -460,6 +466,11 @@ __device__ __forceinline__ void whiten_block(unsigned char *smem, const float *_
         }
     }
     forward_r16(d, v);
+    if (EARLY) {
+        pdl_wait();
+        pdl_trigger();
+        for (int k = t; k < NBIN; k += NT) cp_async4(gs + k, gk + k);
+    }
     cp_async_wait_all();
     __syncthreads();
     float2 o[4][4], ox[4];
@@ -545,7 +556,11 @@ __device__ __forceinline__ WhitenBlock whiten_block_at(const WhitenLayout &L, in
 }
 
 // grid (n_ep * n16, n_det): the blocks on the 16384-point transform, n16 per epoch (bpe, or n_full where the
-// remainder goes to k_whiten_rem); block (e, i) = (blockIdx.x / n16, blockIdx.x % n16)
+// remainder goes to k_whiten_rem); block (e, i) = (blockIdx.x / n16, blockIdx.x % n16).
+// EARLY (one wave of blocks, which find room beside the few CTAs of a short filter build): a programmatic dependent of
+// the build, which triggers once what came before it is complete, so the forward transforms run during the build.
+// Else the gains come in during the forward transform.
+template <bool EARLY>
 __global__ void __launch_bounds__(r16::NT, 2) k_whiten(const float *__restrict__ x, int64_t n, int64_t x_stride,
                                                         const float *__restrict__ gains, int64_t n_psd,
                                                         int64_t out_first, int64_t out_len, int64_t epoch_len, int F,
@@ -559,8 +574,8 @@ __global__ void __launch_bounds__(r16::NT, 2) k_whiten(const float *__restrict__
     const int det = blockIdx.y;
     const int64_t s0 = out_first + b.o - F / 2;  // raw index of block sample 0
     float *dst = y + det * y_stride + b.o;
-    whiten_block(smem_raw, x + det * x_stride + s0, n - s0, gains + ((int64_t)det * n_psd + b.ep) * NBIN, F, b.cnt,
-                 [dst](int64_t q, float v) { dst[q] = v; }, dst);
+    whiten_block<EARLY>(smem_raw, x + det * x_stride + s0, n - s0, gains + ((int64_t)det * n_psd + b.ep) * NBIN, F, b.cnt,
+                        [dst](int64_t q, float v) { dst[q] = v; }, dst);
 }
 
 // grid (n_ep, n_det): each epoch's remainder block on the 4096-point transform (whiten_layout().small_rem).
@@ -571,6 +586,7 @@ __global__ void __launch_bounds__(r16::NT_S) k_whiten_rem(const float *__restric
                                                          int64_t out_first, int64_t out_len, int64_t epoch_len, int F,
                                                          float *__restrict__ y, int64_t y_stride) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_trigger();  // (launched plainly)
     const WhitenLayout L = whiten_layout(out_len, epoch_len, F);
     const WhitenBlock b = whiten_block_at(L, blockIdx.x, L.n_full, out_len, epoch_len, n_psd);
     if (b.cnt <= 0) return;
@@ -713,7 +729,8 @@ bool g_attrs_set = false;
 int set_attrs(afg_ctx *ctx) {
     if (g_attrs_set) return AFG_OK;
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_periodogram, cudaFuncAttributeMaxDynamicSharedMemorySize, WELCH_SMEM));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi_s, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM_S));
     g_attrs_set = true;
@@ -750,6 +767,13 @@ int afg_make_twiddles(afg_ctx *ctx) {
     return set_attrs(ctx);
 }
 
+// the mean over the epochs of n_rows rows of periodograms, a programmatic dependent of their launch
+static cudaError_t launch_psd_mean(const float *P, int64_t n_seg, int seg_step, int K, double *psd, int64_t n_psd, int n_rows,
+                                   cudaStream_t st) {
+    return launch_pdl(k_psd_mean, dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_rows),
+                      dim3(PSD_T), 0, st, P, n_seg, seg_step, K, psd, n_psd);
+}
+
 int launch_psd(afg_ctx *ctx, const float *x, int64_t n, int n_det, int64_t n_psd, int64_t psd_step,
                int64_t psd_span, double *psd, cudaStream_t st, int64_t x_stride) {
     if (x_stride <= 0) x_stride = n;
@@ -770,8 +794,7 @@ int launch_psd(afg_ctx *ctx, const float *x, int64_t n, int n_det, int64_t n_psd
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
         KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_det * (n_seg * 4.0 + n_psd * 8.0) * NBIN);
-        k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), PSD_T, 0, st>>>(
-            P, n_seg, (int)seg_step, (int)K, psd, n_psd);
+        AFG_CUDA(ctx, launch_psd_mean(P, n_seg, (int)seg_step, (int)K, psd, n_psd, n_det, st));
     }
     AFG_LAUNCH_CHECK(ctx, "k_psd_mean");
     return AFG_OK;
@@ -791,14 +814,21 @@ int launch_whiten(afg_ctx *ctx, const float *x, int64_t n, int n_det, const doub
     const int64_t n_ep = wl.bpe > 0 ? wl.n_blocks / wl.bpe : 0;
     const int64_t nb = n_ep * (wl.small_rem ? wl.n_full : wl.bpe);
     if (nb > 0x7fffffff) return afg_fail(ctx, AFG_ERR_ARG, "whiten: too many blocks");
+    // one wave of blocks after a build of few filters: the forward transforms run beside it (64 s span: 98 -> 86 us with
+    // the network's set-up overlapped the same way); a dependent launch of many blocks only took slots (1.38 -> 1.44 ms)
+    const bool early = nb * n_det <= 2 * 152 && (int64_t)n_det * n_psd <= 152;
     {
         // algorithmic: read the cropped span once, write the output once, read the gains
         const double F = ctx->cfg.fir_len;
         KScope ks(ctx, st, KK_WHITEN, 0.0, (double)n_det * ((2.0 * out_len + F - 1.0) * 4.0 + n_psd * NBIN * 4.0));
-        if (nb > 0)
-            k_whiten<<<dim3((unsigned)nb, n_det), r16::NT, WHITEN_SMEM, st>>>(x, n, x_stride, gains, n_psd, out_first,
-                                                                              out_len, epoch_len, ctx->cfg.fir_len, y,
-                                                                              y_stride);
+        if (nb > 0 && early)
+            AFG_CUDA(ctx, launch_pdl(k_whiten<true>, dim3((unsigned)nb, n_det), dim3(r16::NT), WHITEN_SMEM, st, x, n, x_stride,
+                                     (const float *)gains, n_psd, out_first, out_len, epoch_len, (int)ctx->cfg.fir_len, y,
+                                     y_stride));
+        else if (nb > 0)
+            k_whiten<false><<<dim3((unsigned)nb, n_det), r16::NT, WHITEN_SMEM, st>>>(x, n, x_stride, gains, n_psd, out_first,
+                                                                                     out_len, epoch_len, ctx->cfg.fir_len,
+                                                                                     y, y_stride);
     }
     AFG_LAUNCH_CHECK(ctx, "k_whiten");
     if (wl.small_rem && n_ep > 0) {
@@ -837,7 +867,7 @@ int launch_psd_rows(afg_ctx *ctx, const float *const *rows_dev, int n_rows, int6
     AFG_LAUNCH_CHECK(ctx, "k_periodogram");
     {
         KScope ks(ctx, st, KK_PSD_MEAN, 0.0, (double)n_rows * (K * 4.0 + 8.0) * NBIN);
-        k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), 1, (unsigned)n_rows), PSD_T, 0, st>>>(P, K, 0, (int)K, psd, 1);
+        AFG_CUDA(ctx, launch_psd_mean(P, K, 0, (int)K, psd, 1, n_rows, st));
     }
     AFG_LAUNCH_CHECK(ctx, "k_psd_mean");
     return AFG_OK;
@@ -882,9 +912,7 @@ cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, i
                                                                              psd_scale(K, fs));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_psd_mean<<<dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_det), PSD_T, 0, st>>>(
-        P, n_seg, (int)seg_step, (int)K, psd, n_psd);
-    return cudaGetLastError();
+    return launch_psd_mean(P, n_seg, (int)seg_step, (int)K, psd, n_psd, n_det, st);
 }
 
 // Fill the twiddle table and opt the periodogram kernel into its 68 KiB of dynamic shared memory on the
