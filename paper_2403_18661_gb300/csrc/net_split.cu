@@ -6,7 +6,7 @@
 // x_i w_j, each exact in FP32; the six with i + j <= 4 are formed, the other three are below 2^-26 of
 // |x w|.  FP32 SIMT FMAs run at 80 TFLOP/s on this GPU, six BF16 products at 1950 / 6 = 325 (k_conv_fp32
 // of net_fp32.cu, at 78 % of the FP32 pipe, and its GroupNorm took 73.4 ms for 1920 ResNet34 windows and
-// 14.2 ms for 333; this path takes 27.5 and 5.25, and its logits are closer to 64-bit ones: relative error
+// 14.2 ms for 333; this path takes 24.0 and 4.71, and its logits are closer to 64-bit ones: relative error
 // 2.1e-6 against 4.5e-6).
 //
 // Accumulation: the tensor core adds into FP32 but does not promise round-to-nearest, so no long sum is
@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(SC_T, 1) k_conv_split(const SplitConvArgs a) {
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    pdl_trigger();
+    pdl_wait();  // (a programmatic dependent of the GroupNorm before: the set-up overlaps its tail)
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -341,6 +343,8 @@ __global__ void __launch_bounds__(GNS_T, 2) k_gn_split(const float *__restrict__
     const float inv = 1.0f / ((float)L * (float)cg);
     const float *src = raw + (int64_t)c0 * hs + w * hr;
     float v[REG ? GNS_U : 1][8];
+    pdl_trigger();
+    pdl_wait();
 
     // body(i, u, chunk, position) for the warp's units in order
     auto units = [&](auto body) {
@@ -645,6 +649,7 @@ __global__ void k_head_split(const Planes x, int L, int C, const float *__restri
     __shared__ float term[512];
     const int tid = threadIdx.x, nch = C / 8, tpc = 256 / nch, ch = tid % nch, r0 = tid / nch;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    pdl_wait();
     if (r0 < tpc)
         for (int r = r0; r < L; r += tpc) {
             const __nv_bfloat16 *p = x.p + (int64_t)ch * x.cs + plane_row(x, blockIdx.x, r + 1);
@@ -813,7 +818,7 @@ int net_split_reserve(afg_ctx *ctx, int64_t n_win) {
     return split_reserve(ctx, split_chunk(std::max<int64_t>(1, n_win)), act, raw);
 }
 
-static void split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_t nw, cudaStream_t st) {
+static cudaError_t split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_t nw, cudaStream_t st) {
     const ConvLayer &C = ctx->plan.convs[i];
     const SplitPlan &sp = *ctx->splitplan;
     const int tn = tile_rows(C, nw, sp.sms);
@@ -835,16 +840,17 @@ static void split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_
     KScope ks(ctx, st, KK_CONV_SPLIT, 2.0 * nw * C.lout * C.cout * (double)C.k * C.cin,
               4.0 * ((double)nw * ((double)C.lin * C.cin + (double)C.lout * C.cout) + (double)C.k * C.cin * C.cout));
 #define AFG_SPLIT_CONV(TN, MODE) \
-    case TN * 4 + MODE: k_conv_split<TN, MODE><<<grid, SC_T, SplitGeo<TN, MODE>::BYTES, st>>>(a); break;
+    case TN * 4 + MODE: return launch_pdl(k_conv_split<TN, MODE>, dim3(grid), dim3(SC_T), SplitGeo<TN, MODE>::BYTES, st, a);
     switch (tn * 4 + mode_of(C)) {
         AFG_SPLIT_CONV(256, 0) AFG_SPLIT_CONV(256, 1) AFG_SPLIT_CONV(256, 2)
         AFG_SPLIT_CONV(128, 0) AFG_SPLIT_CONV(128, 1) AFG_SPLIT_CONV(128, 2)
         AFG_SPLIT_CONV(64, 0) AFG_SPLIT_CONV(64, 1) AFG_SPLIT_CONV(64, 2)
     }
 #undef AFG_SPLIT_CONV
+    return cudaErrorInvalidValue;  // (not reached)
 }
 
-static void split_gn(afg_ctx *ctx, int i, const float *raw, int64_t nw, const Planes &res, int relu, const Planes &out,
+static cudaError_t split_gn(afg_ctx *ctx, int i, const float *raw, int64_t nw, const Planes &res, int relu, const Planes &out,
                      cudaStream_t st) {
     const ConvLayer &C = ctx->plan.convs[i];
     const int cg = C.cout / ctx->plan.net.groups, nb = (C.lout + 31) / 32;
@@ -856,17 +862,11 @@ static void split_gn(afg_ctx *ctx, int i, const float *raw, int64_t nw, const Pl
     const bool reg = (U + GNS_T / 32 - 1) / (GNS_T / 32) <= GNS_U;
     KScope ks(ctx, st, KK_GROUPNORM, 0.0, (double)nw * C.lout * C.cout * 4.0 * (res.p ? 3.0 : 2.0));
     const dim3 grid(C.cout / cp, (unsigned)nw);
-#define AFG_GN(GS)                                                                                               \
-    do {                                                                                                         \
-        const size_t sm = (size_t)U * (8 / GS) * sizeof(float);                                                  \
-        if (reg) k_gn_split<GS, true><<<grid, GNS_T, sm, st>>>(raw, raw_stride(C, nw), hr, C.lout, cp, lcg, C.gamma, \
-                                                              C.beta, ctx->plan.net.eps, res, relu, out);        \
-        else k_gn_split<GS, false><<<grid, GNS_T, sm, st>>>(raw, raw_stride(C, nw), hr, C.lout, cp, lcg, C.gamma,    \
-                                                           C.beta, ctx->plan.net.eps, res, relu, out);           \
-    } while (0)
-    if (cg >= 8) AFG_GN(8);
-    else if (cg == 4) AFG_GN(4);
-    else AFG_GN(2);
+    const size_t sm = (size_t)U * (8 / std::min(cg, 8)) * sizeof(float);
+#define AFG_GN(GS)                                                                                                        \
+    launch_pdl(reg ? k_gn_split<GS, true> : k_gn_split<GS, false>, grid, dim3(GNS_T), sm, st, raw, raw_stride(C, nw), hr,  \
+               C.lout, cp, lcg, (const float *)C.gamma, (const float *)C.beta, ctx->plan.net.eps, res, relu, out)
+    return cg >= 8 ? AFG_GN(8) : cg == 4 ? AFG_GN(4) : AFG_GN(2);
 #undef AFG_GN
 }
 
@@ -913,24 +913,25 @@ int launch_infer_split(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stri
             const ConvLayer &c1 = P.convs[bp.c1], &c2 = P.convs[bp.c2];
             const bool split_out = b + 1 < P.blocks.size() && P.convs[P.blocks[b + 1].c1].stride == 2;
             const Planes B = make_planes(act[1], nw, c1.lout, c1.cout, false);
-            split_conv(ctx, bp.c1, A, raw, nw, st);
-            split_gn(ctx, bp.c1, raw, nw, none, 1, B, st);
+            AFG_CUDA(ctx, split_conv(ctx, bp.c1, A, raw, nw, st));
+            AFG_CUDA(ctx, split_gn(ctx, bp.c1, raw, nw, none, 1, B, st));
             Planes res = A;
             if (bp.sc >= 0) {
                 res = make_planes(act[3], nw, c2.lout, c2.cout, false);
-                split_conv(ctx, bp.sc, A, raw, nw, st);
-                split_gn(ctx, bp.sc, raw, nw, none, 0, res, st);
+                AFG_CUDA(ctx, split_conv(ctx, bp.sc, A, raw, nw, st));
+                AFG_CUDA(ctx, split_gn(ctx, bp.sc, raw, nw, none, 0, res, st));
             }
-            split_conv(ctx, bp.c2, B, raw, nw, st);
+            AFG_CUDA(ctx, split_conv(ctx, bp.c2, B, raw, nw, st));
             // the output replaces the residual (the same thread reads and writes an element) unless its layout differs
             if (bp.sc >= 0 || split_out) std::swap(ia, ic);
             A = make_planes(act[ia], nw, c2.lout, c2.cout, split_out);
-            split_gn(ctx, bp.c2, raw, nw, res, 1, A, st);
+            AFG_CUDA(ctx, split_gn(ctx, bp.c2, raw, nw, res, 1, A, st));
             AFG_LAUNCH_CHECK(ctx, "residual block (split)");
         }
         {
             KScope ks(ctx, st, KK_HEAD, 2.0 * nw * P.l_last * P.c_last, 4.0 * nw * (double)P.l_last * P.c_last);
-            k_head_split<<<nw, 256, 0, st>>>(A, P.l_last, P.c_last, P.fc_w, P.fc_b, logits, w0);
+            AFG_CUDA(ctx, launch_pdl(k_head_split, dim3(nw), dim3(256), 0, st, A, P.l_last, P.c_last, (const float *)P.fc_w,
+                                     (const float *)P.fc_b, logits, w0));
         }
         AFG_LAUNCH_CHECK(ctx, "k_head_split");
     }

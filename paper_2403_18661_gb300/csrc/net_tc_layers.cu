@@ -366,7 +366,7 @@ __device__ __forceinline__ void ch_store(uint32_t taddr, int p_first, const floa
     }
 }
 
-template <int ORIENT>
+template <int ORIENT, bool PDL>
 __global__ void __launch_bounds__(LT, 1) k_conv_tc(const LayerArgs a) {
     // ORIENT (= a.orient) is compile-time: each instantiation keeps only its own path
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -410,6 +410,10 @@ __global__ void __launch_bounds__(LT, 1) k_conv_tc(const LayerArgs a) {
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    if (PDL) {  // a programmatic dependent of the layer before: everything above, and resident weights, overlap its tail
+        pdl_trigger();
+        if (warp != 0) pdl_wait();
+    }
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -421,6 +425,7 @@ __global__ void __launch_bounds__(LT, 1) k_conv_tc(const LayerArgs a) {
             for (uint32_t o = 0; o < a.w_block_bytes; o += 32768)
                 tc::bulk_load(wsm + o, a.wimg + o, min(32768u, a.w_block_bytes - o), wbar);
         }
+        if (PDL) pdl_wait();
         uint32_t k = 0;  // stage uses
         bool stop = false;
         for (int t = blockIdx.x; t < n_tiles && !stop; t += gridDim.x) {
@@ -1240,6 +1245,7 @@ __global__ void k_head_bf16(const __nv_bfloat16 *__restrict__ x, int L, int C, c
     const int tid = threadIdx.x, nch = C / 8, tpc = 256 / nch;  // threads per chunk
     const int ch = tid % nch, r0 = tid / nch;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    pdl_wait();
     if (r0 < tpc) {
         const uint4 *xc = reinterpret_cast<const uint4 *>(x + ((int64_t)blockIdx.x * nch + ch) * (L + 2) * 8) + 1;
         for (int r = r0; r < L; r += tpc) {
@@ -1499,8 +1505,10 @@ int net_tc_layers_prepare(afg_ctx *ctx) {
         AFG_CUDA(ctx, cudaMemcpy(tp->layers[i].wimg, imgs[i].data(), imgs[i].size() * 2, cudaMemcpyHostToDevice));
         off += (imgs[i].size() * 2 + 1023) / 1024 * 1024;
     }
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
+    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
     {
         const ConvLayer &S = P.convs[0];
         const int smem = (int)stem_tc_smem(ctx->cfg.win_len, S.k, S.lout).total;
@@ -1553,8 +1561,16 @@ static int conv_tc_raw(afg_ctx *ctx, const TcLayer &T, const __nv_bfloat16 *in, 
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
     const unsigned grid = (unsigned)std::max(1, std::min(n_tiles, sms));
-    if (a.orient == 0) k_conv_tc<0><<<grid, LT, layer_smem(a).total, st>>>(a);
-    else k_conv_tc<1><<<grid, LT, layer_smem(a).total, st>>>(a);
+    // Up to 1024 windows a layer is short (7-70 us) and the next one's set-up and resident weights overlap its tail:
+    // 460 -> 382 us for 1 window, 481 -> 397 for 40, 613 -> 580 for 152, 2620 -> 2610 for 900.  Above it the overlap
+    // gains nothing and the wait costs (5169 -> 5205 us for 1900 windows, 10.49 -> 10.65 ms for 4000), even where the
+    // launch is an ordinary one, so the plain kernel is an instantiation of its own.
+    if (nw <= 1024) {
+        AFG_CUDA(ctx, launch_pdl(a.orient == 0 ? k_conv_tc<0, true> : k_conv_tc<1, true>, dim3(grid), dim3(LT), layer_smem(a).total, st, a));
+        return AFG_OK;
+    }
+    if (a.orient == 0) k_conv_tc<0, false><<<grid, LT, layer_smem(a).total, st>>>(a);
+    else k_conv_tc<1, false><<<grid, LT, layer_smem(a).total, st>>>(a);
     AFG_LAUNCH_CHECK(ctx, "k_conv_tc");
     return AFG_OK;
 }
@@ -1814,7 +1830,8 @@ int launch_infer_bf16_full(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_
         }
         {
             KScope ks(ctx, st, KK_HEAD, 2.0 * nw * P.l_last * P.c_last, 2.0 * nw * (double)P.l_last * P.c_last);
-            k_head_bf16<<<nw, 256, 0, st>>>(A, P.l_last, P.c_last, P.fc_w, P.fc_b, logits, w0);
+            AFG_CUDA(ctx, launch_pdl(k_head_bf16, dim3(nw), dim3(256), 0, st, (const __nv_bfloat16 *)A, P.l_last, P.c_last,
+                                     (const float *)P.fc_w, (const float *)P.fc_b, logits, w0));
         }
         AFG_LAUNCH_CHECK(ctx, "k_head_bf16");
     }
