@@ -6,7 +6,7 @@
 // x_i w_j, each exact in FP32; the six with i + j <= 4 are formed, the other three are below 2^-26 of
 // |x w|.  FP32 SIMT FMAs run at 80 TFLOP/s on this GPU, six BF16 products at 1950 / 6 = 325 (k_conv_fp32
 // of net_fp32.cu, at 78 % of the FP32 pipe, and its GroupNorm took 73.4 ms for 1920 ResNet34 windows and
-// 14.2 ms for 333; this path takes 24.0 and 4.71, and its logits are closer to 64-bit ones: relative error
+// 14.2 ms for 333; this path takes 23.9 and 4.47, and its logits are closer to 64-bit ones: relative error
 // 2.1e-6 against 4.5e-6).
 //
 // Accumulation: the tensor core adds into FP32 but does not promise round-to-nearest, so no long sum is
@@ -216,24 +216,36 @@ __global__ void __launch_bounds__(SC_T, 1) k_conv_split(const SplitConvArgs a) {
                 const uint32_t tb = tq + (uint32_t)(buf * 256);
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
-                    if constexpr (COLS >= 32) {
+                    // 32 columns at a time, then the 16 and the 8 that are left
+                    const uint32_t th = tb + ((uint32_t)(16 * hf) << 16);
 #pragma unroll
-                        for (int b = 0; b < COLS / 32; ++b) {
-                            uint32_t r[16];
-                            tc::tmem_ld16x256b_x4_nowait(tb + ((uint32_t)(16 * hf) << 16) + (uint32_t)(32 * b), r);
-                            tc::tmem_wait_ld();
-                            tc::tmem_regs_ready(r);
+                    for (int b = 0; b < COLS / 32; ++b) {
+                        uint32_t r[16];
+                        tc::tmem_ld16x256b_x4_nowait(th + (uint32_t)(32 * b), r);
+                        tc::tmem_wait_ld();
+                        tc::tmem_regs_ready(r);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) acc[hf][16 * b + i] += __uint_as_float(r[i]);
-                        }
-                    } else {
+                        for (int i = 0; i < 16; ++i) acc[hf][16 * b + i] += __uint_as_float(r[i]);
+                    }
+                    if constexpr (COLS % 32 >= 16) {
+                        constexpr int C0 = COLS / 32 * 32;
                         uint32_t r[8];
-                        tc::tmem_ld16x256b_x2_nowait(tb + ((uint32_t)(16 * hf) << 16), r);
+                        tc::tmem_ld16x256b_x2_nowait(th + C0, r);
                         tc::tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(r[i]));  // (uses stay after the wait)
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) acc[hf][i] += __uint_as_float(r[i]);
+                        for (int i = 0; i < 8; ++i) acc[hf][C0 / 2 + i] += __uint_as_float(r[i]);
+                    }
+                    if constexpr (COLS % 16 == 8) {
+                        constexpr int C0 = COLS / 16 * 16;
+                        uint32_t r[4];
+                        tc::tmem_ld16x256b_x1_nowait(th + C0, r);
+                        tc::tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) asm volatile("" : "+r"(r[i]));
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[hf][C0 / 2 + i] += __uint_as_float(r[i]);
                     }
                 }
                 tc::fence_before_sync();
@@ -698,13 +710,25 @@ constexpr int SPLIT_MAX_CHUNK = 1024;
 static int mode_of(const ConvLayer &C) { return C.stride == 1 ? 0 : C.k == 3 ? 1 : 2; }
 static int64_t conv_rows(const ConvLayer &C, int64_t nw) { return nw * (C.lout + (C.stride == 1 ? 2 : 1)); }
 
-// Output rows per tile.  Wide tiles need the fewest shared-memory bytes per MMA; where they would leave
-// half of the SMs without a tile, narrower ones shorten the launch instead.
+// Cycles of one stage of a tile of tn rows: its 6 taps MMAs at 4096 MACs a clock, or (tn < 256, where the weights'
+// 4 KB an MMA are shared by fewer rows) their operand reads and the stage's copies at the 128 B/clk of shared memory.
+static int64_t stage_cycles(int tn, int taps) {
+    return std::max<int64_t>(6 * taps * tn / 2, (6 * taps * (4096 + 32 * tn) + 6 * taps * 2048 + 6 * 16 * tn) / 128);
+}
+
+// Output rows per tile.  Wide tiles cost the fewest cycles a row (9.0 at 256, 9.1 at 224, 9.8 at 192, 12 at 128, 19 at
+// 64 with three taps); narrower ones fill the last wave, or shorten the only one: the width whose waves of one tile an
+// SM take the fewest cycles, the wider one of equals.  Against 256, else 128 or 64 where half of the SMs had no tile:
+// 152 ResNet34 windows 2.32 -> 2.20 ms, 333 4.71 -> 4.47; 960 the same.
 static int tile_rows(const ConvLayer &C, int64_t nw, int sms) {
     const int64_t rows = conv_rows(C, nw), slices = (C.cout + 127) / 128;
-    for (int tn : {256, 128})
-        if ((rows + tn - 1) / tn * slices * 2 > sms) return tn;
-    return 64;
+    int best = 0;
+    int64_t least = 0;
+    for (int tn : {256, 224, 192, 128, 64}) {
+        const int64_t waves = ((rows + tn - 1) / tn * slices + sms - 1) / sms, t = waves * stage_cycles(tn, C.k);
+        if (!best || t < least) best = tn, least = t;
+    }
+    return best;
 }
 
 static bool split_supported(const afg_ctx *ctx) {
@@ -757,6 +781,8 @@ int net_split_prepare(afg_ctx *ctx) {
     AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_split<TN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                        (int)SplitGeo<TN, MODE>::BYTES))
     AFG_SPLIT_ATTR(256, 0); AFG_SPLIT_ATTR(256, 1); AFG_SPLIT_ATTR(256, 2);
+    AFG_SPLIT_ATTR(224, 0); AFG_SPLIT_ATTR(224, 1); AFG_SPLIT_ATTR(224, 2);
+    AFG_SPLIT_ATTR(192, 0); AFG_SPLIT_ATTR(192, 1); AFG_SPLIT_ATTR(192, 2);
     AFG_SPLIT_ATTR(128, 0); AFG_SPLIT_ATTR(128, 1); AFG_SPLIT_ATTR(128, 2);
     AFG_SPLIT_ATTR(64, 0); AFG_SPLIT_ATTR(64, 1); AFG_SPLIT_ATTR(64, 2);
 #undef AFG_SPLIT_ATTR
@@ -794,7 +820,7 @@ static Planes make_planes(__nv_bfloat16 *p, int64_t nw, int L, int C, bool split
     o.ps = (C / 8) * o.cs;
     return o;
 }
-static int64_t raw_stride(const ConvLayer &C, int64_t nw) { return (conv_rows(C, nw) + 255) / 256 * 256; }
+static int64_t raw_stride(const ConvLayer &C, int64_t nw) { return (conv_rows(C, nw) + 224 + 255) / 256 * 256; }  // (whole tiles of any width)
 
 // The workspaces of a launch sequence over nw windows: four activations in planes and one raw output.
 static int split_reserve(afg_ctx *ctx, int64_t nw, __nv_bfloat16 *(&act)[4], float *&raw) {
@@ -843,6 +869,8 @@ static cudaError_t split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw,
     case TN * 4 + MODE: return launch_pdl(k_conv_split<TN, MODE>, dim3(grid), dim3(SC_T), SplitGeo<TN, MODE>::BYTES, st, a);
     switch (tn * 4 + mode_of(C)) {
         AFG_SPLIT_CONV(256, 0) AFG_SPLIT_CONV(256, 1) AFG_SPLIT_CONV(256, 2)
+        AFG_SPLIT_CONV(224, 0) AFG_SPLIT_CONV(224, 1) AFG_SPLIT_CONV(224, 2)
+        AFG_SPLIT_CONV(192, 0) AFG_SPLIT_CONV(192, 1) AFG_SPLIT_CONV(192, 2)
         AFG_SPLIT_CONV(128, 0) AFG_SPLIT_CONV(128, 1) AFG_SPLIT_CONV(128, 2)
         AFG_SPLIT_CONV(64, 0) AFG_SPLIT_CONV(64, 1) AFG_SPLIT_CONV(64, 2)
     }

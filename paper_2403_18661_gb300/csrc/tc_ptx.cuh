@@ -267,6 +267,11 @@ __device__ __forceinline__ void tmem_regs_ready(uint32_t (&r)[16]) {
 // 16 lanes x 8 columns per repetition (the MMA accumulator fragment): thread t receives
 // (lane t/4, columns 2(t%4) and 2(t%4)+1) and (lane 8 + t/4, the same columns) of each
 // 8-column group, group g in r[4g .. 4g + 3]
+__device__ __forceinline__ void tmem_ld16x256b_x1_nowait(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld16x256b_x2_nowait(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])

@@ -62,3 +62,19 @@ def test_split_long_call_and_simt_path_agree():
         ctx.sync()
         ctx.close()
     assert np.max(np.abs(got[0] - got[1]) / (1 + np.abs(got[1]))) <= LOGIT_TOL
+
+
+@pytest.mark.parametrize("n_win", [64, 152])
+def test_split_tile_widths(n_win):
+    """Window counts whose layers, of every stride and kernel, take tiles of 192 (64 windows) and 224 rows (152)."""
+    net, win_len = NETS[0]
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=win_len)
+    w = inputs.make_weights(net, 29)
+    y = np.random.default_rng(n_win).standard_normal((2, (n_win - 1) * 64 + win_len)).astype(np.float32)
+    ctx = abi.Context(wl, w)
+    z = ctx.infer_windows(torch.from_numpy(y).cuda(), 0, 64, n_win).cpu().numpy()
+    ctx.sync()
+    for j in (0, 1, n_win // 3, n_win // 2, n_win - 2, n_win - 1):
+        want = orc.network(net, w, y[:, j * 64:j * 64 + win_len].astype(np.float64))
+        assert abs(z[j] - want) <= LOGIT_TOL * (1 + abs(want)), (j, z[j], want)
+    ctx.close()
