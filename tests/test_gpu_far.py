@@ -126,3 +126,34 @@ def test_trigger_times_match_the_oracle(mode):
     with pytest.raises(abi.AfgError):
         c.trigger_times([wl.n_win - wl.n_int + 1], n_raw=10**7)
     c.close()
+
+
+@pytest.mark.parametrize("n", [1, 4095, 4096, 4097, 8193, 100_003, 1_048_577])
+@pytest.mark.parametrize("kind", ["spread", "equal", "special"])
+def test_far_sort_tile_edges(ctx, n, kind):
+    """One key, whole and ragged tiles of 4096 keys, many tiles; every key in one digit of each pass; infinities, both
+    zeros, NaN and subnormals, sorted by their bits.  Exact; the count lies below the capacity, the rest is untouched."""
+    rng = np.random.default_rng(n)
+    cap = n + 3000 if n < 9000 else n + 1
+    x = rng.standard_normal(cap).astype(np.float32)
+    if kind == "equal":
+        x[:] = 1.25
+        x[::7919] = -3.0
+    elif kind == "special":
+        sp = np.array([np.inf, -np.inf, 0.0, -0.0, np.nan, 1e-42, -1e-42, 3e38], dtype=np.float32)
+        x = sp[rng.integers(0, len(sp), cap)]
+    fg = np.array([0.5], dtype=np.float32)
+    out = (torch.empty(1, dtype=torch.int64, device="cuda"), torch.empty(1, dtype=torch.float64, device="cuda"),
+           torch.full((cap,), 7.5, device="cuda"))
+    n_dev = torch.tensor([n], dtype=torch.int64, device="cuda")
+    for _ in range(2):  # the second call finds the first one's workspaces
+        cnt, _, srt = ctx.far(_dev(x), _dev(fg), 1.0, n_bg=n_dev, bg_cap=cap, out=out)
+    ctx.sync()
+    b = x[:n].view(np.uint32).astype(np.uint64)
+    key = np.where(b >> 31, ~b & 0xFFFFFFFF, b | 0x80000000)  # ascending with the value
+    want = x[:n][np.argsort(0xFFFFFFFF - key, kind="stable")]
+    got = srt.cpu().numpy()
+    assert np.array_equal(got[:n].view(np.uint32), want.view(np.uint32))
+    assert np.all(got[n:] == 7.5)
+    if kind != "special":  # (among NaN the search's order is not a number's)
+        assert cnt.item() == int(np.sum(x[:n] > 0.5))
