@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(GNS_T, 2) k_gn_split(const float *__restrict__
     __shared__ float grstd[256];
     __shared__ __align__(16) float scl[512], shf[512];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t w = blockIdx.y;
+    const int64_t w = gridDim.y - 1 - blockIdx.y;  // (what the convolution wrote last is still in L2: 333 windows -1 %)
     const int c0 = blockIdx.x * cp, nb = (L + 31) / 32, U = cp / 8 * nb, cg = 1 << lcg;
     const int per = (U + NW - 1) / NW, u0 = warp * per, u1 = min(U, u0 + per);
     const int ch0 = u0 / nb, b0 = u0 - ch0 * nb;  // chunk and 32-position block of the warp's first unit
