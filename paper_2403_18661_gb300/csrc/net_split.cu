@@ -6,7 +6,7 @@
 // x_i w_j, each exact in FP32; the six with i + j <= 4 are formed, the other three are below 2^-26 of
 // |x w|.  FP32 SIMT FMAs run at 80 TFLOP/s on this GPU, six BF16 products at 1950 / 6 = 325 (k_conv_fp32
 // of net_fp32.cu, at 78 % of the FP32 pipe, and its GroupNorm took 73.4 ms for 1920 ResNet34 windows and
-// 14.2 ms for 333; this path takes 23.9 and 4.47, and its logits are closer to 64-bit ones: relative error
+// 14.2 ms for 333; this path takes 23.9 and 4.44, and its logits are closer to 64-bit ones: relative error
 // 2.1e-6 against 4.5e-6).
 //
 // Accumulation: the tensor core adds into FP32 but does not promise round-to-nearest, so no long sum is
@@ -75,7 +75,7 @@ __device__ __forceinline__ bool sc_wait(uint64_t *bar, uint32_t parity, int *abo
 
 // One tile: 128 output channels (TMEM lanes) x TN rows (columns).  Per stage the 6 TAPS MMAs of
 // 128 x TN x 16 read 4 KB + 32 TN B of shared memory each, 96 B/clk at TN = 256, and 62 KB are copied in
-// (27 B/clk): under the 128 B/clk of shared memory, so TN = 256 is the tile wherever it fills the GPU.
+// (27 B/clk): under the 128 B/clk of shared memory.  Narrower tiles are chosen by tile_rows.
 template <int TN, int MODE>
 __global__ void __launch_bounds__(SC_T, 1) k_conv_split(const SplitConvArgs a) {
     using G = SplitGeo<TN, MODE>;
