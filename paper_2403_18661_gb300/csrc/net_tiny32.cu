@@ -10,7 +10,9 @@
 //
 // Bound by the FP32 pipe (9 k clocks a layer of 16 -> 16 channels, 3 taps, 1536 positions).  3601 windows: 6.0 ms as
 // one launch per convolution and GroupNorm (each activation written and read through memory, the stem with integer
-// divisions per output), 1.89 ms here.
+// divisions per output), 1.89 ms here.  The FMA pipe is 57 % busy: reductions and the cluster barrier
+// stand between the layers' sums.  Four CTAs of a quarter each, two on an SM: 2.2 ms at best (more reductions per
+// position, and 74 of 76 clusters fit).
 #include <algorithm>
 
 #include "afg_internal.cuh"
