@@ -203,6 +203,7 @@ struct afg_ctx {
     int64_t bytes_held = 0;
     int *d_err = nullptr;             // device-side failure record (bounded waits that gave up)
     Workspace ws[32];
+    bool capturing = false;           // a batch's graph is being captured: the workspaces stay as they are
     float *rs_taps[17] = {};          // decimation filters by factor (resample.cu)
 };
 

@@ -30,10 +30,13 @@ int afg_cuda_fail(afg_ctx *ctx, cudaError_t e, const char *what) {
 
 // Grow-only workspace slot.  Growing frees the old buffer (synchronising
 // the device through cudaFree), so steady-state calls never allocate.
+// Refused while a graph is captured: nodes already captured hold the old buffer.
 int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out) {
     Workspace &w = ctx->ws[slot];
     if (bytes == 0) bytes = 256;
     if (w.bytes < bytes) {
+        if (ctx->capturing)
+            return afg_fail(ctx, AFG_ERR_STATE, "workspace %d: %zu bytes not reserved before the capture", slot, bytes);
         size_t grow = std::max(bytes, w.bytes + w.bytes / 4);
         int64_t after = ctx->bytes_held - (int64_t)w.bytes + (int64_t)grow;
         if (ctx->cfg.hbm_budget > 0 && after > ctx->cfg.hbm_budget) {
@@ -44,7 +47,11 @@ int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out) {
                                 slot, bytes, (long long)ctx->cfg.hbm_budget);
         }
         if (w.p) {
-            cudaFree(w.p);
+            const cudaError_t e = cudaFree(w.p);  // (refused while a caller's own capture is under way: kept then)
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return afg_cuda_fail(ctx, e, "workspace: cudaFree");
+            }
             ctx->bytes_held -= (int64_t)w.bytes;
             w.p = nullptr;
             w.bytes = 0;

@@ -346,8 +346,10 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
     memcpy(f0, ctx->prof.flops, sizeof f0);
     memcpy(b0, ctx->prof.bytes, sizeof b0);
     AFG_CUDA(ctx, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    ctx->capturing = true;
     rc = enqueue(ctx, P, x, x_len, p, segs_dev, series_dev, cnt, psd, white, lg, stat, trig_idx, trig_cap, n_trig,
                  segs_host, st);
+    ctx->capturing = false;
     cudaGraph_t graph_obj = nullptr;
     cudaError_t e = cudaStreamEndCapture(st, &graph_obj);
     if (rc) {

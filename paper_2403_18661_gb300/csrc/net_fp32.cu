@@ -653,7 +653,7 @@ static int64_t simt_chunk(const afg_ctx *ctx, int64_t n_win) {
     return std::min<int64_t>(chunk, 16384);
 }
 
-// Reserve what launch_infer_fp32 over n_win windows uses (a graph capture allows no allocation).
+// Reserve what launch_infer_fp32 over up to n_win windows uses (a graph capture allows no allocation).
 int infer_fp32_reserve(afg_ctx *ctx, int64_t n_win) {
     if (net_split_available(ctx)) return net_split_reserve(ctx, n_win);
     if (net_tiny32_fits(ctx)) return AFG_OK;  // (no workspaces)

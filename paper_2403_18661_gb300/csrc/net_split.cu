@@ -838,10 +838,12 @@ static int split_reserve(afg_ctx *ctx, int64_t nw, __nv_bfloat16 *(&act)[4], flo
     return rc;
 }
 
+// What any call of up to n_win windows uses.  (Not the sequence of n_win itself: 1025 windows go in sequences of 513,
+// but 1024 in one.)
 int net_split_reserve(afg_ctx *ctx, int64_t n_win) {
     __nv_bfloat16 *act[4];
     float *raw;
-    return split_reserve(ctx, split_chunk(std::max<int64_t>(1, n_win)), act, raw);
+    return split_reserve(ctx, std::min<int64_t>(std::max<int64_t>(1, n_win), SPLIT_MAX_CHUNK), act, raw);
 }
 
 static cudaError_t split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_t nw, cudaStream_t st) {

@@ -227,3 +227,53 @@ def test_batch_full_day_sampled(capsys):
         print(f"\nfull-day batch: {tw} windows, {len(tr)} triggers; {checked} sampled windows of "
               f"{len(picks)} segments x 4 timeslides vs the oracle, max |dz|/(1+|z|) = {worst:.3e}")
     ctx.close()
+
+
+@pytest.mark.parametrize("order", [(0, 1), (1, 0)])
+def test_batch_graph_of_wide_fp32_series_around_the_sequence_length(order):
+    """A captured batch of FP32 wide-network series on both sides of the 1024 windows a launch sequence holds (1022 in
+    one sequence, 2115 in three of 705): every workspace is reserved before the capture, and capture and replays equal
+    the direct call and the series on their own."""
+    import dataclasses
+    net = inputs.NetSpec(stem_k=3, stem_stride=2, stem_pool=1, widths=(64,), blocks=(1,), groups=16)
+    wl = dataclasses.replace(inputs.TIMESLIDE_DAY, net=net, stride=15, win_len=1056)
+    lengths = [wl.psd_len + wl.crop + n * wl.epoch_len + 100 for n in (1, 2)]
+    x = (1e-21 * np.random.default_rng(3).standard_normal((2, sum(lengths)))).astype(np.float32)
+    segs = [(0, lengths[0]), (lengths[0], lengths[1])]
+    segs = [segs[i] for i in order]
+    w = inputs.make_weights(net, 7)
+    xd = torch.from_numpy(x).cuda()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    ctx = abi.Context(wl, w)
+    n_win, _, _ = ctx.batch_layout(segs, 2, SHIFT_STEP)
+    assert sorted(n_win) == [1022, 2115]
+    with torch.cuda.stream(s):  # the first call of the context
+        out = ctx.batch_run(xd, segs, 2, SHIFT_STEP, use_graph=True, stream=s)
+        s.synchronize()
+        first = [t.clone() for t in out]
+        out[0].zero_()
+        out = ctx.batch_run(xd, segs, 2, SHIFT_STEP, use_graph=True, out=out, stream=s)
+        s.synchronize()
+    ctx.sync()
+    n_trig = int(first[3])
+    assert torch.equal(out[0], first[0]) and torch.equal(out[1], first[1]) and int(out[3]) == n_trig
+    direct = abi.Context(wl, w)
+    d = direct.batch_run(xd, segs, 2, SHIFT_STEP)
+    torch.cuda.synchronize()
+    for a, b in zip(d[:2], first):
+        assert torch.equal(a, b)
+    assert int(d[3]) == n_trig and torch.equal(d[2][:n_trig], first[2][:n_trig])
+    lo = 0
+    for (off, n), nw in zip(segs, n_win):
+        xs = xd[:, off:off + n].contiguous()
+        n_ep = (n - wl.psd_len - wl.crop) // wl.epoch_len
+        psd = direct.psd_estimate(xs, n_psd=n_ep, psd_step=wl.epoch_len, psd_span=wl.psd_len)
+        y = direct.whiten(xs, psd, wl.psd_len, n_ep * wl.epoch_len, epoch_len=wl.epoch_len)
+        for k in (1, 2):
+            z = direct.infer_windows(y, 0, wl.stride, nw, shift=k * SHIFT_STEP)
+            assert torch.equal(z, first[0][lo:lo + nw])
+            lo += nw
+    direct.sync()
+    for c in (ctx, direct):
+        c.close()
