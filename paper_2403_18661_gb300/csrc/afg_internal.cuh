@@ -203,6 +203,7 @@ struct afg_ctx {
     int64_t bytes_held = 0;
     int *d_err = nullptr;             // device-side failure record (bounded waits that gave up)
     Workspace ws[32];
+    int64_t ws_moves = 0;             // workspaces that were freed and allocated anew
     bool capturing = false;           // a batch's graph is being captured: the workspaces stay as they are
     float *rs_taps[17] = {};          // decimation filters by factor (resample.cu)
 };
@@ -225,6 +226,8 @@ enum {
     WS_SCAN,
     WS_BATCH_SEGS,
     WS_BATCH_SERIES,
+    WS_GRAPH_SEGS,   // descriptors of the captured batch: a direct call leaves them alone
+    WS_GRAPH_SERIES,
     WS_FAR_KEYS,
     WS_FAR_HIST,
     WS_FAR_SORTED,

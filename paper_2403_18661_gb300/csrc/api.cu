@@ -55,6 +55,7 @@ int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out) {
             ctx->bytes_held -= (int64_t)w.bytes;
             w.p = nullptr;
             w.bytes = 0;
+            ++ctx->ws_moves;
         }
         void *p = nullptr;
         cudaError_t e = cudaMalloc(&p, grow);

@@ -173,6 +173,7 @@ struct GraphKey {
     afg_batch_params p;
     uint64_t seg_hash;
     int n_seg;
+    int64_t ws_moves;  // the nodes hold workspace pointers
 };
 
 uint64_t hash_segs(const afg_segment *s, int n) {
@@ -284,6 +285,7 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
         const GraphKey &k = ctx->batch->g.key;
         if (k.x == x && k.logits == logits && k.stat == stat && k.trig == trig_idx && k.ntrig == n_trig &&
             k.stream == stream && k.x_len == x_len && k.trig_cap == trig_cap && k.n_seg == n_seg &&
+            k.ws_moves == ctx->ws_moves &&
             memcmp(&k.p, p, sizeof *p) == 0 && k.seg_hash == hash_segs(segs_host, n_seg)) {
             AFG_CUDA(ctx, cudaGraphLaunch(ctx->batch->g.exec, st));
             for (int i = 0; i < KK_COUNT; ++i) {
@@ -313,10 +315,12 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
     if (!rc) rc = afg_ws_reserve(ctx, WS_PERIODOGRAM, periodogram_bytes(2 * P.max_nseg), &tmp);
     if (!rc) rc = afg_ws_reserve(ctx, WS_FILTER, (size_t)2 * P.max_ep * NBIN * sizeof(float), &tmp);
     if (!rc && !lg) rc = afg_ws_reserve(ctx, WS_LOGITS, (size_t)P.total_win * sizeof(float), (void **)&lg);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_BATCH_SEGS, P.segs.size() * sizeof(SegDesc), (void **)&segs_dev);
+    if (!rc)
+        rc = afg_ws_reserve(ctx, graph ? WS_GRAPH_SEGS : WS_BATCH_SEGS, P.segs.size() * sizeof(SegDesc), (void **)&segs_dev);
     const size_t ser_bytes = P.series.size() * sizeof(SeriesDesc);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_BATCH_SERIES, ser_bytes + P.series.size() * sizeof(int64_t) + 256,
-                                 (void **)&series_dev);
+    if (!rc)
+        rc = afg_ws_reserve(ctx, graph ? WS_GRAPH_SERIES : WS_BATCH_SERIES,
+                            ser_bytes + P.series.size() * sizeof(int64_t) + 256, (void **)&series_dev);
     if (rc) return rc;
     int64_t *cnt = reinterpret_cast<int64_t *>(reinterpret_cast<char *>(series_dev) + ((ser_bytes + 255) / 256) * 256);
     if (ctx->cfg.precision == AFG_FP32) {
@@ -326,6 +330,7 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
         rc = infer_fp32_reserve(ctx, max_win);
         if (rc) return rc;
     }
+    if (graph && ctx->batch) ctx->batch->g.valid = false;  // (its descriptors are replaced)
     // descriptors are uploaded synchronously: they are constant for a captured graph
     AFG_CUDA(ctx, cudaMemcpy(segs_dev, P.segs.data(), P.segs.size() * sizeof(SegDesc), cudaMemcpyHostToDevice));
     AFG_CUDA(ctx, cudaMemcpy(series_dev, P.series.data(), ser_bytes, cudaMemcpyHostToDevice));
@@ -366,7 +371,7 @@ extern "C" int afg_batch_run(afg_ctx *ctx, const float *x, int64_t x_len, const 
         g.bytes[i] = ctx->prof.bytes[i] - b0[i];
     }
     g.key = GraphKey{x, logits, stat, trig_idx, n_trig, stream, x_len, trig_cap, *p, hash_segs(segs_host, n_seg),
-                     n_seg};
+                     n_seg, ctx->ws_moves};
     g.valid = true;
     AFG_CUDA(ctx, cudaGraphLaunch(g.exec, st));
     return AFG_OK;

@@ -277,3 +277,36 @@ def test_batch_graph_of_wide_fp32_series_around_the_sequence_length(order):
     direct.sync()
     for c in (ctx, direct):
         c.close()
+
+
+def test_batch_graph_after_other_calls_of_the_context():
+    """A captured batch, then direct calls that replace what its nodes refer to (the descriptors by a batch of other
+    segments of the same sizes; the workspaces by a longer batch), then the captured call again: the first result each
+    time."""
+    wl = inputs.TIMESLIDE_DAY
+    n = wl.psd_len + wl.crop + wl.epoch_len * np.array([1, 3, 6]) + 50
+    x = (1e-21 * np.random.default_rng(4).standard_normal((2, int(n.sum()) + n[0]))).astype(np.float32)
+    off = np.concatenate([[0], np.cumsum(n)])
+    a, b = [(int(off[0]), int(n[0])), (int(off[1]), int(n[1]))], [(int(off[1]) + 700, int(n[1])), (int(off[2]), int(n[0]))]
+    big = [(int(off[2]), int(n[2])), (int(off[1]), int(n[1]))]
+    w = inputs.make_weights(wl.net, wl.weight_seed)
+    xd = torch.from_numpy(x).cuda()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    for precision in (abi.AFG_BF16, abi.AFG_FP32):
+        ctx = abi.Context(wl, w, precision=precision)
+        with torch.cuda.stream(s):
+            out = ctx.batch_run(xd, a, 2, SHIFT_STEP, use_graph=True, stream=s)
+            s.synchronize()
+            first = [t.clone() for t in out]
+            n_trig = int(first[3])
+            for other in (b, big, b):
+                ctx.batch_run(xd, other, 2, SHIFT_STEP, stream=s)
+                s.synchronize()
+                out[0].zero_(), out[1].zero_()
+                out = ctx.batch_run(xd, a, 2, SHIFT_STEP, use_graph=True, out=out, stream=s)
+                s.synchronize()
+                assert torch.equal(out[0], first[0]) and torch.equal(out[1], first[1]) and int(out[3]) == n_trig
+                assert torch.equal(out[2][:n_trig], first[2][:n_trig])
+        ctx.sync()
+        ctx.close()
