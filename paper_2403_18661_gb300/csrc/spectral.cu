@@ -10,7 +10,7 @@
 //                     scaling of the segment's spectrum, stored as FP32 with
 //                     the segment's exponent
 //   k_psd_mean        sum over the K segments of each epoch in pairs of floats
-//                     (FP64 where segments are too many or too far apart),
+//                     (FP64 where segments are too many or too far apart in power),
 //                     a run of epochs per thread
 //   k_whiten          one 8192-output overlap-save block per CTA: FP32 real
 //                     FFT of 8192 + F - 1 samples (zero padded to NFFT),
@@ -241,8 +241,11 @@ __device__ __forceinline__ double pair_double(float ah, float al, int e) {
 // prefix sums of the 64 s PSDs kept that pipe 81 % busy.  For those (step 2, 15 segments) an epoch is a tree
 // over shared partial sums: with A_i = P_2i + P_2i+1, B_i = A_i + A_i+1, C_i = B_i + B_i+2, epoch e is
 // C_e + B_e+4 + A_e+6 + P_2e+14, six pair additions.  Other short sums are formed directly; long ones, and runs
-// whose exponents differ by more than 80 (a segment 2^40 times another), slide an FP64 sum.
+// whose exponents differ by more than 80 (a segment 2^40 times another), slide an FP64 sum: the segments that enter
+// are added and those that leave subtracted.  An error stays in that sum at the size of the largest it has been, so
+// where it has fallen by 2^8 (a much louder segment left) or is no longer finite it is formed afresh.
 constexpr int PSD_SEGS = 512;  // segments of a run the pair sums hold scales for
+constexpr int PSD_CANCEL = 8 << 20;  // 2^8 in the high word of a double
 
 // A thread takes bins k and k + PSD_T as the halves of packed additions (the loads and stores of both coalesce).
 constexpr int PSD_T = 128;
@@ -348,12 +351,25 @@ __global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P,
             const float *r = src + s * PER_ROW;
             return scaled_double(r[kk], __float_as_int(r[PER_EXP - k]));
         };
-        double acc = 0.0;
-        for (int q = 0; q < K; ++q) acc += val(q);
+        auto afresh = [&](int64_t s) {
+            double a = 0.0;
+            for (int q = 0; q < K; ++q) a += val(s + q);
+            return a;
+        };
+        double acc = afresh(0);
+        int top = __double2hiint(acc);  // of the largest sum since the last fresh one (non-negative doubles order as ints)
         dst[kk] = acc;
         for (int64_t i = 1; i < n_e; ++i) {
             const int64_t s_old = (i - 1) * seg_step, s_new = s_old + K;
-            for (int q = 0; q < seg_step; ++q) acc += val(s_new + q) - val(s_old + q);
+            for (int q = 0; q < seg_step; ++q) {
+                acc += val(s_new + q) - val(s_old + q);
+                top = max(top, __double2hiint(acc));
+            }
+            const int hi = __double2hiint(acc);
+            if (hi < top - PSD_CANCEL || hi >= 0x7FF00000) {
+                acc = afresh(i * seg_step);
+                top = __double2hiint(acc);
+            }
             dst[i * NBIN + kk] = acc;
         }
     }

@@ -36,3 +36,27 @@ def test_epoch_sums_match_single_periodograms(k_seg, seg_step, kind, n_psd):
     want = np.stack([one[:, e * seg_step:e * seg_step + k_seg].mean(axis=1) for e in range(n_psd)], axis=1)
     assert np.all(np.abs(got - want) <= RTOL * want)
     ctx.close()
+
+
+@pytest.mark.parametrize("k_seg,seg_step", [(15, 2), (15, 1), (4, 3), (3, 5), (16, 16), (31, 2), (20, 7)])
+@pytest.mark.parametrize("kind", ["loud", "nan"])
+@pytest.mark.parametrize("where", ["first", "middle"])
+def test_epochs_around_an_outlying_segment(k_seg, seg_step, kind, where):
+    """A segment 2^100 times the others in power, or of NaN, at the start or in the middle of a run of epochs: the epochs
+    that hold it are its sums, and those before and after it have none of it."""
+    n_psd = 45
+    n_seg = (n_psd - 1) * seg_step + k_seg
+    n = (n_seg - 1) * HOP + NFFT
+    x = (1e-21 * np.random.default_rng(n_seg).standard_normal((2, n))).astype(np.float32)
+    a = 0 if where == "first" else n_seg // 2 * HOP + 100
+    x[:, a:a + HOP] = np.nan if kind == "nan" else x[:, a:a + HOP] * np.float32(2.0 ** 50)
+    wl = inputs.PLAIN_64S
+    ctx = abi.Context(wl, inputs.make_weights(wl.net, 1))
+    xd = torch.from_numpy(x).cuda()
+    one = ctx.psd_estimate(xd, n_psd=n_seg, psd_step=HOP, psd_span=NFFT).cpu().numpy()
+    got = ctx.psd_estimate(xd, n_psd=n_psd, psd_step=seg_step * HOP, psd_span=(k_seg - 1) * HOP + NFFT).cpu().numpy()
+    want = np.stack([one[:, e * seg_step:e * seg_step + k_seg].mean(axis=1) for e in range(n_psd)], axis=1)
+    finite = np.isfinite(want)
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    assert finite.any() and np.all(np.abs(got[finite] - want[finite]) <= RTOL * want[finite])
+    ctx.close()
