@@ -216,8 +216,10 @@ __device__ __forceinline__ Pair2 psum(float2 a, float2 b) {
     const float2 s = __fadd2_rn(a, b), t = sub2(s, a);
     return {s, __fadd2_rn(sub2(a, sub2(s, t)), sub2(b, t))};
 }
-// The double (h + l) 2^e from its bits: the low part as an integer of the high part's last double place.
+// The double (h + l) 2^e from its bits: the low part as an integer of the high part's last double place.  (A sum with
+// an infinity in it: the high part is infinite, the low one NaN from inf - inf.)
 __device__ __forceinline__ double pair_double(float ah, float al, int e) {
+    if (isinf(ah)) return scaled_double(ah, e);
     const float h = __fadd_rn(ah, al), l = __fsub_rn(al, __fsub_rn(h, ah));
     const uint32_t u = __float_as_uint(h), E = u >> 23;
     if (E - 1u >= 253u) return scaled_double(h, e);  // zero, (nearly) infinite or NaN

@@ -60,3 +60,34 @@ def test_epochs_around_an_outlying_segment(k_seg, seg_step, kind, where):
     assert np.array_equal(np.isnan(got), np.isnan(want))
     assert finite.any() and np.all(np.abs(got[finite] - want[finite]) <= RTOL * want[finite])
     ctx.close()
+
+
+@pytest.mark.parametrize("k_seg,seg_step", [(1, 1), (15, 2), (4, 3), (31, 2)])
+def test_overflowing_spectrum_is_infinite(k_seg, seg_step):
+    """A tone of 5e34 in one segment: its squares, scaled to the spectrum's finite part, are past FP32's range.  The
+    epochs that hold the segment are infinite, not NaN, at the bins far from the tone and from its partner in the
+    half-length transform (8192 - 1000, where infinities are subtracted), and the others are as they were."""
+    n_psd, hit = 12, 7
+    n_seg = (n_psd - 1) * seg_step + k_seg
+    n = (n_seg - 1) * HOP + NFFT
+    x = (1e-21 * np.random.default_rng(n_seg).standard_normal((1, n))).astype(np.float32)
+    wl = inputs.PLAIN_64S
+    ctx = abi.Context(wl, inputs.make_weights(wl.net, 1))
+
+    def psd():
+        return ctx.psd_estimate(torch.from_numpy(x).cuda(), n_psd=n_psd, psd_step=seg_step * HOP,
+                                psd_span=(k_seg - 1) * HOP + NFFT).cpu().numpy()[0]
+
+    quiet = psd()
+    a = hit * seg_step * HOP
+    x[0, a:a + NFFT] = 5e34 * np.cos(2 * np.pi * 1000 * np.arange(NFFT) / NFFT)
+    got = psd()
+    # segments that share samples with the tone
+    seg = [s for s in range(n_seg) if abs(s * HOP - a) < NFFT]
+    for e in range(n_psd):
+        own = range(e * seg_step, e * seg_step + k_seg)
+        if a // HOP in own:
+            assert np.all(np.isinf(got[e, 2000:7000]))
+        elif not set(own) & set(seg):
+            assert np.all(np.abs(got[e] - quiet[e]) <= RTOL * quiet[e])
+    ctx.close()
