@@ -161,7 +161,8 @@ int afg_wait_check(afg_ctx *ctx, int64_t limit_ns, int32_t n_blocks, int64_t *wa
  * transformed with a real FFT in FP32, squared in FP32 after an exact
  * power-of-two scaling of the segment's spectrum (so that no square under- or
  * overflows; relative rounding 1.2e-7) and summed in pairs of floats (about 46
- * bits; in FP64 for more than 16 segments or segments 2^40 apart):
+ * bits; in FP64 for more than 16 segments, for 8 or more times the segments
+ * between epochs, and where segments are 2^40 apart):
  *   psd[d][e][k] = c_k / (K fs sum w^2) sum_s |X_s(k)|^2, k in [0, nfft/2],
  *   c_k = 1 for k = 0 and k = nfft/2, else 2.
  * x: [n_det][n] float32.  psd: [n_det][n_psd][nfft/2+1] float64.

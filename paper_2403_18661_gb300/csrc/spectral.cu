@@ -10,8 +10,9 @@
 //                     scaling of the segment's spectrum, stored as FP32 with
 //                     the segment's exponent
 //   k_psd_mean        sum over the K segments of each epoch in pairs of floats
-//                     (FP64 where segments are too many or too far apart in power),
-//                     a run of epochs per thread
+//                     (FP64 where segments are too far apart in power), a run of
+//                     epochs per thread
+//   k_psd_mean64      the same in FP64, for many segments or a short step
 //   k_whiten          one 8192-output overlap-save block per CTA: FP32 real
 //                     FFT of 8192 + F - 1 samples (zero padded to NFFT),
 //                     multiply by the epoch's gains, inverse FFT, keep the
@@ -192,10 +193,11 @@ __global__ void __launch_bounds__(r16::NT, 2) k_periodogram(const float *__restr
 
 // The double u 2^e, bit by bit (no FP64 instruction); u zero, normal, infinite or NaN.
 __device__ __forceinline__ double scaled_double(float v, int e) {
-    const uint32_t u = __float_as_uint(v), E = u >> 23, m23 = u & 0x7FFFFFu;
-    if (E == 0) return 0.0;
-    if (E == 255) return __hiloint2double((int)(0x7FF00000u | (m23 ? 0x80000u : 0u)), 0);
-    return __hiloint2double((int)((uint32_t)((int)E + 896 + e) << 20 | (m23 >> 3)), (int)((m23 & 7u) << 29));
+    const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
+    uint32_t hi = (u >> 3) + ((uint32_t)(896 + e) << 20), lo = u << 29;
+    if (u >= 0x7F800000u) hi = 0x7FF00000u | (u & 0x7FFFFFu ? 0x80000u : 0u), lo = 0u;
+    if (u < 0x00800000u) hi = lo = 0u;
+    return __hiloint2double((int)hi, (int)lo);
 }
 
 // Two sums of non-negative floats (two bins) as h + l (l a few roundings of h at most), in packed instructions
@@ -219,10 +221,9 @@ __device__ __forceinline__ Pair2 psum(float2 a, float2 b) {
 // The double (h + l) 2^e from its bits: the low part as an integer of the high part's last double place.  (A sum with
 // an infinity in it: the high part is infinite, the low one NaN from inf - inf.)
 __device__ __forceinline__ double pair_double(float ah, float al, int e) {
-    if (isinf(ah)) return scaled_double(ah, e);
     const float h = __fadd_rn(ah, al), l = __fsub_rn(al, __fsub_rn(h, ah));
     const uint32_t u = __float_as_uint(h), E = u >> 23;
-    if (E - 1u >= 253u) return scaled_double(h, e);  // zero, (nearly) infinite or NaN
+    if (E - 1u >= 253u) return scaled_double(isinf(ah) ? ah : h, e);  // zero, (nearly) infinite or NaN
     const int li = __float2int_rn(l * __uint_as_float((254 - E) << 23) * 0x1p52f);  // |l| <= half a place of h: < 2^28
     // mantissa 2^52 (1.m) + li in two words
     uint32_t lo = (u << 29) + (uint32_t)li;
@@ -236,19 +237,106 @@ __device__ __forceinline__ double pair_double(float ah, float al, int e) {
     return __hiloint2double((int)(((uint32_t)ed << 20) + hi), (int)lo);
 }
 
+// The epochs [0, n_e) of one bin in FP64: column src of a run's rows (the row's exponent is src[exp]) into dst.
+// The sum slides: the segments that enter are added and those that leave subtracted.  An error stays in the sum at the
+// size of the largest it has been, so where it has fallen by 2^8 (a much louder segment left) or is no longer finite it
+// is formed afresh.  Bound by FP64 additions (16 clk a warp and SM, 63 clk from one to the next) where the runs are many, by
+// the latency of the loads where they are few: those of B terms are in flight together, one bin a thread and blocks of
+// 64 (two bins a thread, a term at a time: 258 us for one PSD of 439 segments, 592 for 40 at step 8; so 47 and 97).
+constexpr int PSD_CANCEL = 8 << 20;  // 2^8 in the high word of a double
+
+// K terms from row src on, in order
+__device__ __noinline__ double psd_sum64(const float *src, int exp, int K) {
+    constexpr int B = 16;
+    double a = 0.0;
+    for (int q = 0; q < K; q += B, src += B * PER_ROW) {
+        float v[B];
+        int e[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            const float *r = src + min(i, K - 1 - q) * PER_ROW;
+            v[i] = r[0];
+            e[i] = __float_as_int(r[exp]);
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+            if (q + i < K) a += scaled_double(v[i], e[i]);
+    }
+    return a;
+}
+
+__device__ __forceinline__ void psd_run64(const float *src, int exp, int seg_step, int K, double *dst, int n_e) {
+    constexpr int B = 8;
+    if (seg_step >= K) {  // no segment is shared
+        for (int i = 0; i < n_e; ++i) dst[(int64_t)i * NBIN] = psd_sum64(src + (int64_t)i * seg_step * PER_ROW, exp, K);
+        return;
+    }
+    double acc = psd_sum64(src, exp, K);
+    *dst = acc;
+    int top = __double2hiint(acc);  // of the largest sum since the last fresh one (non-negative doubles order as ints)
+    const int n = (n_e - 1) * seg_step;  // slides by one segment; epoch i is reached after i seg_step
+    const int64_t ahead = (int64_t)K * PER_ROW;
+    int left = seg_step;
+    for (int j = 0; j < n; j += B, src += B * PER_ROW) {
+        float in[B], out[B];
+        int ei[B], eo[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const float *r = src + min(b, n - 1 - j) * PER_ROW;
+            out[b] = r[0];
+            eo[b] = __float_as_int(r[exp]);
+            in[b] = r[ahead];
+            ei[b] = __float_as_int(r[ahead + exp]);
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            if (j + b >= n) return;
+            acc += scaled_double(in[b], ei[b]) - scaled_double(out[b], eo[b]);
+            const int hi = __double2hiint(acc);
+            top = max(top, hi);
+            if (--left == 0) {
+                left = seg_step;
+                dst += NBIN;
+                if (hi < top - PSD_CANCEL || hi >= 0x7FF00000) {
+                    acc = psd_sum64(src + (b + 1) * PER_ROW, exp, K);
+                    top = __double2hiint(acc);
+                }
+                *dst = acc;
+            }
+        }
+    }
+}
+
+constexpr int PSD_SEGS = 512;  // segments of a run the pair sums hold scales for
+
+// Sums in pairs of floats (else in FP64): up to 16 segments, whose run's scales fit, and fewer than 8 times the step
+// (else the slide's few FP64 additions are less than K pair additions an epoch, as 113 us against 88 for 500 epochs of
+// 15 segments at step 1 and 158 for either at 16 and 2).
+inline bool psd_pairs(int64_t n_psd, int64_t seg_step, int64_t K) {
+    return K <= 16 && (n_psd == 1 || K < 8 * seg_step) && (std::min<int64_t>(PSD_EPT, n_psd) - 1) * seg_step + K <= PSD_SEGS;
+}
+
+// grid (ceil(NBIN / PSD_T64), ceil(n_psd / PSD_EPT), n_det): epochs as FP64 sums
+constexpr int PSD_T64 = 64;
+
+__global__ void __launch_bounds__(PSD_T64) k_psd_mean64(const float *P, int64_t n_seg, int seg_step, int K, double *psd,
+                                                        int64_t n_psd) {
+    const int k = blockIdx.x * PSD_T64 + threadIdx.x;
+    const int64_t e0 = (int64_t)blockIdx.y * PSD_EPT;
+    pdl_trigger();  // (launched plainly)
+    if (k >= NBIN) return;
+    psd_run64(P + ((int64_t)blockIdx.z * n_seg + e0 * seg_step) * PER_ROW + k, PER_EXP - k, seg_step, K,
+              psd + ((int64_t)blockIdx.z * n_psd + e0) * NBIN + k, (int)min((int64_t)PSD_EPT, n_psd - e0));
+}
+
 // grid (ceil(NBIN / 2 PSD_T), ceil(n_psd / PSD_EPT), n_det): the bins of epochs [e0, e0 + PSD_EPT) as sums of the
 // periodograms (already scaled by the density factor; epoch e sums segments [e seg_step, e seg_step + K)).
 // The sums are pairs of floats over the run's largest exponent (about 46 bits; the terms have 24 and an FP32
 // transform's error) and only the result is a double: this GPU retires 2 FP64 adds a clock and SM, and the FP64
 // prefix sums of the 64 s PSDs kept that pipe 81 % busy.  For those (step 2, 15 segments) an epoch is a tree
 // over shared partial sums: with A_i = P_2i + P_2i+1, B_i = A_i + A_i+1, C_i = B_i + B_i+2, epoch e is
-// C_e + B_e+4 + A_e+6 + P_2e+14, six pair additions.  Other short sums are formed directly; long ones, and runs
-// whose exponents differ by more than 80 (a segment 2^40 times another), slide an FP64 sum: the segments that enter
-// are added and those that leave subtracted.  An error stays in that sum at the size of the largest it has been, so
-// where it has fallen by 2^8 (a much louder segment left) or is no longer finite it is formed afresh.
-constexpr int PSD_SEGS = 512;  // segments of a run the pair sums hold scales for
-constexpr int PSD_CANCEL = 8 << 20;  // 2^8 in the high word of a double
-
+// C_e + B_e+4 + A_e+6 + P_2e+14, six pair additions.  Other short sums (psd_pairs) are formed directly; runs
+// whose exponents differ by more than 80 (a segment 2^40 times another) in FP64.
 // A thread takes bins k and k + PSD_T as the halves of packed additions (the loads and stores of both coalesce).
 constexpr int PSD_T = 128;
 
@@ -264,8 +352,8 @@ __global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P,
     const int64_t ns = (int64_t)(n_e - 1) * seg_step + K;
     pdl_wait();
     pdl_trigger();
-    bool pairs = K <= 16 && ns <= PSD_SEGS;
-    if (pairs) {
+    bool pairs;
+    {
         if (tid == 0) {
             elo = 1 << 20;
             ehi = -(1 << 20);
@@ -347,33 +435,15 @@ __global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P,
         }
         return;
     }
-    for (int h = 0; h < (second ? 2 : 1); ++h) {
-        const int kk = h ? PSD_T : 0;
-        auto val = [&](int64_t s) {
-            const float *r = src + s * PER_ROW;
-            return scaled_double(r[kk], __float_as_int(r[PER_EXP - k]));
-        };
-        auto afresh = [&](int64_t s) {
-            double a = 0.0;
-            for (int q = 0; q < K; ++q) a += val(s + q);
-            return a;
-        };
-        double acc = afresh(0);
-        int top = __double2hiint(acc);  // of the largest sum since the last fresh one (non-negative doubles order as ints)
-        dst[kk] = acc;
-        for (int64_t i = 1; i < n_e; ++i) {
-            const int64_t s_old = (i - 1) * seg_step, s_new = s_old + K;
-            for (int q = 0; q < seg_step; ++q) {
-                acc += val(s_new + q) - val(s_old + q);
-                top = max(top, __double2hiint(acc));
-            }
-            const int hi = __double2hiint(acc);
-            if (hi < top - PSD_CANCEL || hi >= 0x7FF00000) {
-                acc = afresh(i * seg_step);
-                top = __double2hiint(acc);
-            }
-            dst[i * NBIN + kk] = acc;
-        }
+    // (psd_run64's code beside the pair sums takes them from 71 registers to 96 and a fifth of their rate)
+#pragma unroll 1
+    for (int i = 0; i < n_e * (second ? 2 : 1); ++i) {
+        const int e = second ? i >> 1 : i, kk = second && (i & 1) ? PSD_T : 0;
+        const float *r = src + (int64_t)e * seg_step * PER_ROW;
+        double a = 0.0;
+#pragma unroll 4
+        for (int q = 0; q < K; ++q, r += PER_ROW) a += scaled_double(r[kk], __float_as_int(r[PER_EXP - k]));
+        dst[(int64_t)e * NBIN + kk] = a;
     }
 }
 
@@ -788,6 +858,13 @@ int afg_make_twiddles(afg_ctx *ctx) {
 // the mean over the epochs of n_rows rows of periodograms, a programmatic dependent of their launch
 static cudaError_t launch_psd_mean(const float *P, int64_t n_seg, int seg_step, int K, double *psd, int64_t n_psd, int n_rows,
                                    cudaStream_t st) {
+    if (!psd_pairs(n_psd, seg_step, K)) {
+        // (launched plainly: early blocks crowd the first SMs that fall free, and those SMs' FP64 pipes: one PSD of 439
+        // segments 102 us, 47 so)
+        k_psd_mean64<<<dim3((NBIN + PSD_T64 - 1) / PSD_T64, (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_rows), PSD_T64, 0, st>>>(
+            P, n_seg, seg_step, K, psd, n_psd);
+        return cudaGetLastError();
+    }
     return launch_pdl(k_psd_mean, dim3((NBIN + 2 * PSD_T - 1) / (2 * PSD_T), (unsigned)((n_psd + PSD_EPT - 1) / PSD_EPT), n_rows),
                       dim3(PSD_T), 0, st, P, n_seg, seg_step, K, psd, n_psd);
 }

@@ -91,3 +91,19 @@ def test_overflowing_spectrum_is_infinite(k_seg, seg_step):
         elif not set(own) & set(seg):
             assert np.all(np.abs(got[e] - quiet[e]) <= RTOL * quiet[e])
     ctx.close()
+
+
+@pytest.mark.parametrize("k_seg,seg_step", [(17, 1), (32, 5), (33, 32), (16, 2), (8, 1), (40, 40), (3, 40), (16, 33)])
+@pytest.mark.parametrize("n_psd", [1, 2, 5, 33])
+def test_fp64_sums_at_batch_edges(k_seg, seg_step, n_psd):
+    """Layouts that sum in FP64: slides and sums that end inside a batch of 8 or 16 terms, steps that share no segment."""
+    n_seg = (n_psd - 1) * seg_step + k_seg
+    x = (1e-21 * np.random.default_rng(n_seg).standard_normal((1, (n_seg - 1) * HOP + NFFT))).astype(np.float32)
+    wl = inputs.PLAIN_64S
+    ctx = abi.Context(wl, inputs.make_weights(wl.net, 1))
+    xd = torch.from_numpy(x).cuda()
+    one = ctx.psd_estimate(xd, n_psd=n_seg, psd_step=HOP, psd_span=NFFT).cpu().numpy()
+    got = ctx.psd_estimate(xd, n_psd=n_psd, psd_step=seg_step * HOP, psd_span=(k_seg - 1) * HOP + NFFT).cpu().numpy()
+    want = np.stack([one[:, e * seg_step:e * seg_step + k_seg].mean(axis=1) for e in range(n_psd)], axis=1)
+    assert np.all(np.abs(got - want) <= RTOL * want)
+    ctx.close()
