@@ -257,8 +257,19 @@ __global__ void __launch_bounds__(RS_T) k_rs_pass(const KeySource src, uint32_t 
     }
 }
 
-// count = #{sorted > x}: the first index whose value is <= x in the decreasing array.  One warp per x: each step
-// splits the range in 33 at 32 probes.
+// count = #{sorted > x}: the first index whose value is <= x in the decreasing array, by bisection
+__device__ __forceinline__ int64_t bisect(const float *sorted, int64_t n, float x) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (sorted[mid] > x) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// One warp per x: each step splits the range in 33 at 32 probes, which is where bisection ends as long as the probes
+// above x are the first ones.  Positive NaN come before every number and are not above it: then each lane bisects.
 __global__ void k_far_count(const float *__restrict__ sorted, const int64_t *n_dev, int64_t cap,
                             const float *__restrict__ fg, int64_t n_fg, double livetime, int64_t *__restrict__ n_above,
                             double *__restrict__ far) {
@@ -266,9 +277,10 @@ __global__ void k_far_count(const float *__restrict__ sorted, const int64_t *n_d
     const int64_t n = dev_count(n_dev, cap);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    const bool nan = n > 0 && isnan(sorted[0]);
     for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; j < n_fg; j += warps) {
         const float x = fg[j];
-        int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
+        int64_t lo = nan ? bisect(sorted, n, x) : 0, hi = nan ? lo : n;  // the answer lies in [lo, hi]
         while (lo < hi) {
             const int64_t step = (hi - lo + 32) / 33, i = lo + step * (lane + 1) - 1;  // probes, in order
             const uint32_t above = __ballot_sync(0xffffffffu, i < hi && sorted[i] > x);

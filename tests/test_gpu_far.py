@@ -157,3 +157,29 @@ def test_far_sort_tile_edges(ctx, n, kind):
     assert np.all(got[n:] == 7.5)
     if kind != "special":  # (among NaN the search's order is not a number's)
         assert cnt.item() == int(np.sum(x[:n] > 0.5))
+
+
+def _bisect(srt, x):
+    lo, hi = 0, len(srt)
+    while lo < hi:
+        mid = (lo + hi) // 2
+        if srt[mid] > x:
+            lo = mid + 1
+        else:
+            hi = mid
+    return lo
+
+
+@pytest.mark.parametrize("n,n_nan", [(1, 1), (33, 1), (40, 39), (5000, 3), (100_003, 700), (100_003, 60_000)])
+def test_far_count_with_nan_in_the_background(ctx, n, n_nan):
+    """Positive NaN sort before every number and negative ones after: the count is where bisection of the sorted
+    background ends, as it is without them."""
+    rng = np.random.default_rng(n + n_nan)
+    bg = np.round(rng.standard_normal(n), 3).astype(np.float32)
+    bg[rng.permutation(n)[:n_nan]] = np.nan
+    bg[rng.permutation(n)[:n // 50]] = np.float32(-np.nan)
+    fg = np.concatenate([rng.standard_normal(200).astype(np.float32) * 2,
+                         np.array([np.nan, np.inf, -np.inf, 0.0, -10.0], dtype=np.float32)])
+    cnt, far, srt = _check(ctx, bg, fg, 7.0)
+    assert list(cnt) == [_bisect(srt[:n], x) for x in fg]
+    assert np.array_equal(far, cnt / 7.0)
