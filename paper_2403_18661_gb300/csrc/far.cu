@@ -8,8 +8,8 @@
 // are the keys of lower digits (from the counts) plus those of its digit in the tiles before it, which it adds up
 // from the sums the tiles publish (decoupled look-back, Merrill & Garland 2016).  The first pass reads the
 // statistics, the last writes them.  Launches are sized by the capacity; only the tiles that hold keys do work.
-// Each foreground statistic x then gets count = #{background > x} by a 32-way search (one warp), and
-// FAR = count / livetime.  The background count may live on the device (as afg_batch_run writes it), so
+// Each foreground statistic x then gets count = #{background > x} by a 32-way search (one warp; one thread's bisection
+// where there are many) and FAR = count / livetime.  The background count may live on the device (as afg_batch_run writes it), so
 // every kernel reads n = min(*n_dev, cap) itself and nothing synchronises.
 // A handful of small kernels in a row: latency sets the time (0.93 million events: 330 us with the histogram scanned
 // by one block and four barriers per 256 keys of the scatter; 97 us as histogram, row scan and scatter a pass, 13
@@ -296,6 +296,23 @@ __global__ void k_far_count(const float *__restrict__ sorted, const int64_t *n_d
     }
 }
 
+// One thread per x.  A warp per x has a quarter of the dependent loads but as many loads in all as eight threads, so
+// above about a warp an x that the GPU holds at once (8192) the loads bind it.  With the sort, 0.93 million background
+// events: 4096 x 69 us either way, 65,536 101 us as warps and 77 so, a million 595 and 105 (4000 events, a million x: 541
+// and 42).
+__global__ void k_far_bisect(const float *sorted, const int64_t *n_dev, int64_t cap, const float *fg, int64_t n_fg,
+                             double livetime, int64_t *n_above, double *far) {
+    pdl_wait();
+    const int64_t n = dev_count(n_dev, cap), threads = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_fg; j += threads) {
+        const int64_t c = bisect(sorted, n, fg[j]);
+        if (n_above) n_above[j] = c;
+        if (far) far[j] = (double)c / livetime;
+    }
+}
+
+constexpr int64_t FAR_WARPS = 8192;  // foreground events searched by a warp each
+
 }  // namespace
 
 int launch_far(afg_ctx *ctx, const float *bg_stat, const int64_t *bg_idx, const int64_t *n_bg_dev, int64_t bg_cap,
@@ -330,7 +347,10 @@ int launch_far(afg_ctx *ctx, const float *bg_stat, const int64_t *bg_idx, const 
                                      n_bg_dev, bg_cap, pass, (const uint32_t *)hist, ticket, status, ctx->d_err));
             src.keys = ko;
         }
-        if (n_fg > 0)
+        if (n_fg > FAR_WARPS)
+            AFG_CUDA(ctx, launch_pdl(k_far_bisect, dim3((unsigned)std::min<int64_t>((n_fg + 255) / 256, 152 * 16)), dim3(256), 0,
+                                     st, (const float *)bg_sorted, n_bg_dev, bg_cap, fg, n_fg, livetime_s, n_above, far));
+        else if (n_fg > 0)
             AFG_CUDA(ctx, launch_pdl(k_far_count, dim3((unsigned)std::min<int64_t>((n_fg + 7) / 8, 152 * 16)), dim3(256), 0, st,
                                      (const float *)bg_sorted, n_bg_dev, bg_cap, fg, n_fg, livetime_s, n_above, far));
     }

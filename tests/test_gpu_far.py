@@ -183,3 +183,17 @@ def test_far_count_with_nan_in_the_background(ctx, n, n_nan):
     cnt, far, srt = _check(ctx, bg, fg, 7.0)
     assert list(cnt) == [_bisect(srt[:n], x) for x in fg]
     assert np.array_equal(far, cnt / 7.0)
+
+
+@pytest.mark.parametrize("n_fg", [8192, 8193, 100_001])
+@pytest.mark.parametrize("n", [1, 5000, 60_001])
+def test_far_count_of_many_foreground_events(ctx, n, n_fg):
+    """Both sides of the number of events from which each is searched by one thread, not by one warp."""
+    rng = np.random.default_rng(n + n_fg)
+    bg = np.round(rng.standard_normal(n), 2).astype(np.float32)
+    fg = np.round(rng.standard_normal(n_fg) * 2, 2).astype(np.float32)
+    fg[-1] = np.nan
+    cnt, far, _ = _check(ctx, bg, fg, 3.0)
+    want = n - np.searchsorted(np.sort(bg), fg, side="right")
+    want[-1] = 0  # nothing is above a NaN
+    assert np.array_equal(cnt, want) and np.array_equal(far, want / 3.0)
