@@ -12,8 +12,8 @@
 // (O(log h) an index), flags and their count; k_cluster_write turns the flags into indices.
 // One launch for a series of one tile, two for longer ones (before: one launch for the
 // statistic and one for each doubling, each a pass over memory: 10 launches and 75 us for
-// 1.4 million windows at h = 64, now 2 and 15 us).  Integrations or clusters too long for a tile take the
-// separate passes below.
+// 1.4 million windows at h = 64, now 2 and 15 us).  Integrations too long for a tile are a launch of their own
+// before it; clusters too long for a tile take the separate passes below.
 #include <math.h>
 
 #include <algorithm>
@@ -52,8 +52,10 @@ __device__ __forceinline__ float max_nan(float a, float b) {  // NaN if either i
     return d;
 }
 
+// z: logits, or (stat null, n_int 1) the statistic itself.
 // NAN_STOPS (series of at most CL_DIRECT indices, half-widths up to CL_DIRECT_H): an index with a NaN within h of it
-// is no trigger, and a side without any index is no condition; else NaNs count as -inf, and so do missing sides.
+// is no trigger, and a side without any index is no condition; else NaNs count as -inf unless a whole side is NaN (then
+// no trigger), and so do missing sides.
 constexpr int64_t CL_DIRECT = 16384;
 constexpr int CL_DIRECT_H = 256;
 
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(CL_T) k_cluster(const float *__restrict__ z, i
             float s = 0.f;
             for (int q = 0; q < n_int; ++q) s += zl[i + q];
             v = s / (float)n_int;
-            if (i >= h && i < h + CL_N) stat[j] = v;
+            if (stat && i >= h && i < h + CL_N) stat[j] = v;
         }
         A[i] = v;
     }
@@ -263,7 +265,8 @@ int launch_integrate(afg_ctx *ctx, const float *logits, int64_t n_win, int n_int
     const int64_t n_out = n_win - n_int + 1;
     const int h = cluster_half;
     const int64_t tiles = (n_out + CL_N - 1) / CL_N;
-    if (n_out > 0 && h <= CL_H && n_int <= CL_INT && tiles <= 0x7fffffff) {
+    if (n_out > 0 && h <= CL_H && tiles <= 0x7fffffff) {
+        const bool apart = n_int > CL_INT;  // statistic first
         void *pf = nullptr, *pc = nullptr;
         if (tiles > 1) {
             int rc = afg_ws_reserve(ctx, WS_TRIG_FLAG, (size_t)tiles * 32 * sizeof(uint32_t), &pf);
@@ -274,9 +277,11 @@ int launch_integrate(afg_ctx *ctx, const float *logits, int64_t n_win, int n_int
         int *counts = static_cast<int *>(pc);
         {
             KScope ks(ctx, st, KK_INTEGRATE, (double)n_out * n_int, (double)(n_win + n_out) * 4.0);
-            const size_t sm = cluster_smem(h, n_int);
+            if (apart) k_integrate<<<(unsigned)((n_out + 255) / 256), 256, 0, st>>>(logits, n_out, n_int, stat);
+            const int ni = apart ? 1 : n_int;
             AFG_CUDA(ctx, launch_pdl(n_out <= CL_DIRECT && h <= CL_DIRECT_H ? k_cluster<true> : k_cluster<false>,
-                                     dim3((unsigned)tiles), dim3(CL_T), sm, st, logits, n_out, (int)n_int, h, stat, flags,
+                                     dim3((unsigned)tiles), dim3(CL_T), cluster_smem(h, ni), st,
+                                     (const float *)(apart ? stat : logits), n_out, ni, h, apart ? nullptr : stat, flags,
                                      counts, trig_idx, trig_cap, n_trig));
         }
         AFG_LAUNCH_CHECK(ctx, "k_cluster");

@@ -74,3 +74,27 @@ def test_more_tiles_than_a_block_adds_up(ctx):
     want = torch.nonzero((z > left) & (z >= right))[:, 0]
     assert torch.equal(stat, z) and int(cnt) == want.numel()
     assert torch.equal(idx[:want.numel()], want)
+
+
+@pytest.mark.parametrize("n_out,h,n_int", [(1, 0, 1025), (700, 0, 1500), (1500, 8, 1025), (5000, 256, 2048), (5000, 257, 2048),
+                                           (16384, 64, 1025), (16385, 64, 1025)])
+def test_long_integrations(ctx, n_out, h, n_int):
+    """Integrations past a tile's, with NaN and -inf in some of the statistics only: a short series keeps its rule for
+    both (a NaN neighbour stops a trigger, a missing side is no condition); in a long one a whole side of NaN stops it."""
+    rng = np.random.default_rng(n_out + h)
+    z = rng.standard_normal(n_out + n_int - 1).astype(np.float32)
+    z[min(9, n_out - 1)] = -np.inf      # the first statistics: -inf
+    if n_out > 100:
+        z[n_int + n_out // 2] = np.nan  # statistics from n_out / 2 + 1 on, at most n_int of them
+    with np.errstate(invalid="ignore"):
+        want = _stat(z, n_int)
+        trig = _triggers(want, h)
+    if not (n_out <= 16384 and h <= 256):
+        nan = np.isnan(want)
+        trig = np.array([j for j in trig if not (j >= h and nan[j - h:j].all()) and
+                         not (j + h < n_out and nan[j + 1:j + h + 1].all())], dtype=np.int64)
+    assert np.isfinite(want).any() or n_out == 1
+    stat, idx, n = ctx.integrate(torch.from_numpy(z).cuda(), n_int, h, trig_cap=max(len(trig), 1))
+    assert np.array_equal(stat.cpu().numpy(), want, equal_nan=True)
+    assert int(n) == len(trig)
+    assert np.array_equal(idx.cpu().numpy()[:len(trig)], trig)
