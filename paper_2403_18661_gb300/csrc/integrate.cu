@@ -12,8 +12,8 @@
 // (O(log h) an index), flags and their count; k_cluster_write turns the flags into indices.
 // One launch for a series of one tile, two for longer ones (before: one launch for the
 // statistic and one for each doubling, each a pass over memory: 10 launches and 75 us for
-// 1.4 million windows at h = 64, now 2 and 15 us).  Integrations too long for a tile are a launch of their own
-// before it; clusters too long for a tile take the separate passes below.
+// 1.4 million windows at h = 64, now 2 and 15 us).  Long integrations may be a launch of their own
+// before it (launch_integrate); clusters too long for a tile take the separate passes below.
 #include <math.h>
 
 #include <algorithm>
@@ -266,7 +266,10 @@ int launch_integrate(afg_ctx *ctx, const float *logits, int64_t n_win, int n_int
     const int h = cluster_half;
     const int64_t tiles = (n_out + CL_N - 1) / CL_N;
     if (n_out > 0 && h <= CL_H && tiles <= 0x7fffffff) {
-        const bool apart = n_int > CL_INT;  // statistic first
+        // The statistic first: integrations past a tile's, and long ones where a tile would form the sums of h > 256
+        // indices to each side again (1.4 million windows, 1024 each: 234 us apart or together at h = 256, 249 and 459 at
+        // 1024; 128 each: 58 and 82).  Short integrations stay together, a launch less.
+        const bool apart = n_int > CL_INT || (h > 256 && n_int >= 128);
         void *pf = nullptr, *pc = nullptr;
         if (tiles > 1) {
             int rc = afg_ws_reserve(ctx, WS_TRIG_FLAG, (size_t)tiles * 32 * sizeof(uint32_t), &pf);

@@ -98,3 +98,15 @@ def test_long_integrations(ctx, n_out, h, n_int):
     assert np.array_equal(stat.cpu().numpy(), want, equal_nan=True)
     assert int(n) == len(trig)
     assert np.array_equal(idx.cpu().numpy()[:len(trig)], trig)
+
+
+@pytest.mark.parametrize("n_out,h,n_int", [(700, 256, 128), (700, 257, 127), (700, 257, 128), (3000, 1024, 128),
+                                           (20000, 300, 1024)])
+def test_long_integrations_beside_long_clusters(ctx, n_out, h, n_int):
+    """Both sides of the rule that forms the statistic before the clustering."""
+    z = np.random.default_rng(n_int + h).standard_normal(n_out + n_int - 1).astype(np.float32)
+    want = _stat(z, n_int)
+    trig = _triggers(want, h)
+    stat, idx, n = ctx.integrate(torch.from_numpy(z).cuda(), n_int, h, trig_cap=max(len(trig), 1))
+    assert np.array_equal(stat.cpu().numpy(), want)
+    assert int(n) == len(trig) and np.array_equal(idx.cpu().numpy()[:len(trig)], trig)
