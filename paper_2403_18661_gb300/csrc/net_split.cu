@@ -700,12 +700,14 @@ struct SplitPlan {
     std::vector<unsigned char *> wimg;  // indexed like NetPlan::convs (0 unused)
     void *mem = nullptr;
     int sms = 0;
+    int64_t max_chunk = 1;  // windows per launch sequence at most
 };
 
-// Windows per launch sequence at most (1.4 GB of ResNet34 activations).  Each of the 70 launches costs about
-// 5 us whatever its size, and a short sequence leaves its last wave of tiles part empty: 1920 ResNet34
+// Windows per launch sequence at most (1.4 GB of ResNet34 activations), and bytes of each of its five buffers, which
+// hold fewer of the longest and widest windows.  Each of the 70 launches costs about 5 us whatever its size, and a short sequence leaves its last wave of tiles part empty: 1920 ResNet34
 // windows took 33.4 ms in sequences of 98 (activations stay in L2), 29.0 of 392, 27.4 of 960, 27.6 of 1920.
-constexpr int SPLIT_MAX_CHUNK = 1024;
+constexpr int64_t SPLIT_MAX_CHUNK = 1024;
+constexpr int64_t SPLIT_MAX_BYTES = (int64_t)4 << 30;
 
 static int mode_of(const ConvLayer &C) { return C.stride == 1 ? 0 : C.k == 3 ? 1 : 2; }
 static int64_t conv_rows(const ConvLayer &C, int64_t nw) { return nw * (C.lout + (C.stride == 1 ? 2 : 1)); }
@@ -729,6 +731,34 @@ static int tile_rows(const ConvLayer &C, int64_t nw, int sms) {
         if (!best || t < least) best = tn, least = t;
     }
     return best;
+}
+
+static Planes make_planes(__nv_bfloat16 *p, int64_t nw, int L, int C, bool split) {
+    Planes o;
+    o.p = p;
+    o.rows = split ? L / 2 + 1 : L + 2;
+    const int64_t r = nw * o.rows + SC_SLACK;
+    o.odd = split ? r * 8 : 0;
+    o.cs = (split ? 2 : 1) * r * 8;
+    o.ps = (C / 8) * o.cs;
+    return o;
+}
+// (whole tiles of any width)
+static int64_t raw_stride(const ConvLayer &C, int64_t nw) { return (conv_rows(C, nw) + 224 + 255) / 256 * 256; }
+
+// Bytes of each of the four activation buffers (three planes) and of the raw output of a sequence of nw windows
+static void split_bytes(const NetPlan &P, int64_t nw, int64_t &planes, int64_t &raw) {
+    planes = 3 * make_planes(nullptr, nw, P.l_after_stem, P.convs[0].cout, false).ps;
+    raw = 0;
+    for (size_t i = 1; i < P.convs.size(); ++i) {
+        const ConvLayer &C = P.convs[i];
+        for (bool split : {false, true})
+            if (!split || C.lout % 2 == 0)
+                planes = std::max(planes, 3 * make_planes(nullptr, nw, C.lout, C.cout, split).ps);
+        raw = std::max(raw, (int64_t)C.cout * raw_stride(C, nw));
+    }
+    planes *= (int64_t)sizeof(__nv_bfloat16);
+    raw *= (int64_t)sizeof(float);
 }
 
 static bool split_supported(const afg_ctx *ctx) {
@@ -769,6 +799,11 @@ int net_split_prepare(afg_ctx *ctx) {
     ctx->splitplan = sp;
     ctx->bytes_held += (int64_t)total;
     AFG_CUDA(ctx, cudaMemset(d, 0, total));
+    sp->max_chunk = SPLIT_MAX_CHUNK;
+    for (int64_t planes, raw; sp->max_chunk > 1; sp->max_chunk = sp->max_chunk * 3 / 4) {
+        split_bytes(P, sp->max_chunk, planes, raw);
+        if (std::max(planes, raw) <= SPLIT_MAX_BYTES) break;
+    }
     sp->wimg.resize(P.convs.size());
     for (size_t i = 1; i < P.convs.size(); ++i) {
         const ConvLayer &C = P.convs[i];
@@ -804,37 +839,19 @@ void net_split_release(afg_ctx *ctx) {
 
 bool net_split_available(const afg_ctx *ctx) { return ctx->splitplan != nullptr; }
 
-// Windows per launch sequence for a call of n_win: equal shares of at most SPLIT_MAX_CHUNK
-static int64_t split_chunk(int64_t n_win) {
-    const int64_t n = (n_win + SPLIT_MAX_CHUNK - 1) / SPLIT_MAX_CHUNK;
+// Windows per launch sequence for a call of n_win: equal shares
+static int64_t split_chunk(const afg_ctx *ctx, int64_t n_win) {
+    const int64_t n = (n_win + ctx->splitplan->max_chunk - 1) / ctx->splitplan->max_chunk;
     return (n_win + n - 1) / n;
 }
 
-static Planes make_planes(__nv_bfloat16 *p, int64_t nw, int L, int C, bool split) {
-    Planes o;
-    o.p = p;
-    o.rows = split ? L / 2 + 1 : L + 2;
-    const int64_t r = nw * o.rows + SC_SLACK;
-    o.odd = split ? r * 8 : 0;
-    o.cs = (split ? 2 : 1) * r * 8;
-    o.ps = (C / 8) * o.cs;
-    return o;
-}
-static int64_t raw_stride(const ConvLayer &C, int64_t nw) { return (conv_rows(C, nw) + 224 + 255) / 256 * 256; }  // (whole tiles of any width)
-
 // The workspaces of a launch sequence over nw windows: four activations in planes and one raw output.
 static int split_reserve(afg_ctx *ctx, int64_t nw, __nv_bfloat16 *(&act)[4], float *&raw) {
-    const NetPlan &P = ctx->plan;
-    int64_t pl = 3 * make_planes(nullptr, nw, P.l_after_stem, P.convs[0].cout, false).ps, rw = 0;
-    for (size_t i = 1; i < P.convs.size(); ++i) {
-        const ConvLayer &C = P.convs[i];
-        for (bool split : {false, true})
-            if (!split || C.lout % 2 == 0) pl = std::max(pl, 3 * make_planes(nullptr, nw, C.lout, C.cout, split).ps);
-        rw = std::max(rw, (int64_t)C.cout * raw_stride(C, nw));
-    }
+    int64_t planes, rw;
+    split_bytes(ctx->plan, nw, planes, rw);
     int rc = AFG_OK;
-    for (int i = 0; i < 4 && !rc; ++i) rc = afg_ws_reserve(ctx, WS_ACT0 + i, (size_t)pl * 2, (void **)&act[i]);
-    if (!rc) rc = afg_ws_reserve(ctx, WS_RAW, (size_t)rw * 4, (void **)&raw);
+    for (int i = 0; i < 4 && !rc; ++i) rc = afg_ws_reserve(ctx, WS_ACT0 + i, (size_t)planes, (void **)&act[i]);
+    if (!rc) rc = afg_ws_reserve(ctx, WS_RAW, (size_t)rw, (void **)&raw);
     return rc;
 }
 
@@ -843,7 +860,7 @@ static int split_reserve(afg_ctx *ctx, int64_t nw, __nv_bfloat16 *(&act)[4], flo
 int net_split_reserve(afg_ctx *ctx, int64_t n_win) {
     __nv_bfloat16 *act[4];
     float *raw;
-    return split_reserve(ctx, std::min<int64_t>(std::max<int64_t>(1, n_win), SPLIT_MAX_CHUNK), act, raw);
+    return split_reserve(ctx, std::min<int64_t>(std::max<int64_t>(1, n_win), ctx->splitplan->max_chunk), act, raw);
 }
 
 static cudaError_t split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_t nw, cudaStream_t st) {
@@ -906,7 +923,7 @@ int launch_infer_split(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stri
     const NetPlan &P = ctx->plan;
     const ConvLayer &S = P.convs[0];
     const int W = ctx->cfg.win_len;
-    const int64_t chunk = split_chunk(n_win);
+    const int64_t chunk = split_chunk(ctx, n_win);
     __nv_bfloat16 *act[4];
     float *raw;
     int rc = split_reserve(ctx, chunk, act, raw);

@@ -78,3 +78,23 @@ def test_split_tile_widths(n_win):
         want = orc.network(net, w, y[:, j * 64:j * 64 + win_len].astype(np.float64))
         assert abs(z[j] - want) <= LOGIT_TOL * (1 + abs(want)), (j, z[j], want)
     ctx.close()
+
+
+def test_split_buffers_stay_under_4_gib():
+    """The largest window and width an accepted network can have: 50 MB of activations a window, so that 1024 windows
+    would take 51 GB a buffer.  The call goes in shorter sequences, and its logits are those of short calls."""
+    net = inputs.NetSpec(stem_k=3, stem_stride=1, stem_pool=0, widths=(512,), blocks=(1,), groups=32)
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=16384)
+    w = inputs.make_weights(net, 3)
+    n_win, stride = 200, 64
+    y = torch.randn((2, (n_win - 1) * stride + 16384), device="cuda", generator=torch.Generator("cuda").manual_seed(9))
+    ctx = abi.Context(wl, w)
+    z = ctx.infer_windows(y, 0, stride, n_win)
+    ctx.sync()
+    assert ctx.bytes_held <= 5 * (4 << 30) + (64 << 20)
+    few = abi.Context(wl, w)
+    for a in (0, 100, 197):
+        assert torch.equal(few.infer_windows(y, a * stride, stride, 3), z[a:a + 3])
+    few.sync()
+    for c in (ctx, few):
+        c.close()
