@@ -294,6 +294,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 int afg_fail(afg_ctx *ctx, int code, const char *fmt, ...);
 int afg_cuda_fail(afg_ctx *ctx, cudaError_t e, const char *what);
 int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out);
+void afg_ws_release(afg_ctx *ctx, int slot);
 void batch_cache_release(afg_ctx *ctx);
 void serve_release(afg_ctx *ctx);
 

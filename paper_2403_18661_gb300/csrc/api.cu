@@ -61,8 +61,8 @@ int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out) {
         cudaError_t e = cudaMalloc(&p, grow);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return afg_fail(ctx, AFG_ERR_OOM, "workspace %d: cudaMalloc(%zu) failed: %s", slot, grow,
-                            cudaGetErrorString(e));
+            const int code = e == cudaErrorMemoryAllocation ? AFG_ERR_OOM : AFG_ERR_CUDA;  // (no room, or a caller's capture)
+            return afg_fail(ctx, code, "workspace %d: cudaMalloc(%zu) failed: %s", slot, grow, cudaGetErrorString(e));
         }
         w.p = p;
         w.bytes = grow;
@@ -70,6 +70,14 @@ int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out) {
     }
     *out = w.p;
     return AFG_OK;
+}
+
+void afg_ws_release(afg_ctx *ctx, int slot) {
+    Workspace &w = ctx->ws[slot];
+    if (!w.p || ctx->capturing || cudaFree(w.p) != cudaSuccess) return;
+    ctx->bytes_held -= (int64_t)w.bytes;
+    w = Workspace();
+    ++ctx->ws_moves;
 }
 
 void prof_release(afg_ctx *ctx);

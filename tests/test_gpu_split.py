@@ -98,3 +98,28 @@ def test_split_buffers_stay_under_4_gib():
     few.sync()
     for c in (ctx, few):
         c.close()
+
+
+def test_split_on_a_device_with_little_room():
+    """Room for a fraction of a launch sequence's buffers (18 GB for this network): shorter sequences, the same logits."""
+    net = inputs.NetSpec(stem_k=3, stem_stride=1, stem_pool=0, widths=(512,), blocks=(1,), groups=32)
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=16384)
+    w = inputs.make_weights(net, 3)
+    n_win, stride = 60, 64
+    y = torch.randn((2, (n_win - 1) * stride + 16384), device="cuda", generator=torch.Generator("cuda").manual_seed(9))
+    ctx = abi.Context(wl, w)
+    want = ctx.infer_windows(y, 0, stride, n_win)
+    ctx.sync()
+    ctx.close()
+    ctx = abi.Context(wl, w)
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (5 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        for _ in range(2):
+            assert torch.equal(ctx.infer_windows(y, 0, stride, n_win), want)
+        ctx.sync()
+        assert ctx.bytes_held < 5 << 30
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    ctx.close()
