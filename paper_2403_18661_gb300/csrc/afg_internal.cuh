@@ -254,6 +254,9 @@ struct KScope {
 // returns once that kernel has completed and its writes are visible.
 // pdl_trigger() in the earlier kernel lets the dependent launch start early.
 // Both are no-ops for kernels launched without the attribute.
+// What the kernel before writes is not constant while this one runs: a kernel
+// with pdl_wait() takes it through plain pointers and loads, no
+// const __restrict__ and no __ldg, which may be moved ahead of the wait.
 // ----------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -270,9 +270,8 @@ __device__ __forceinline__ int64_t bisect(const float *sorted, int64_t n, float 
 
 // One warp per x: each step splits the range in 33 at 32 probes, which is where bisection ends as long as the probes
 // above x are the first ones.  Positive NaN come before every number and are not above it: then each lane bisects.
-__global__ void k_far_count(const float *__restrict__ sorted, const int64_t *n_dev, int64_t cap,
-                            const float *__restrict__ fg, int64_t n_fg, double livetime, int64_t *__restrict__ n_above,
-                            double *__restrict__ far) {
+__global__ void k_far_count(const float *sorted, const int64_t *n_dev, int64_t cap, const float *fg, int64_t n_fg,
+                            double livetime, int64_t *__restrict__ n_above, double *__restrict__ far) {
     pdl_wait();
     const int64_t n = dev_count(n_dev, cap);
     const int lane = threadIdx.x & 31;

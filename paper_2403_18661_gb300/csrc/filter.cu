@@ -488,7 +488,7 @@ __device__ __forceinline__ void st_cluster(float2 *local, int rank, float2 v) { 
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y) : "memory");
 }
 
-__global__ void __launch_bounds__(FGT) k_filter_one(const double *__restrict__ psd, int k_hp,
+__global__ void __launch_bounds__(FGT) k_filter_one(const double *psd, int k_hp,
                                                                              const float2 *__restrict__ tap,
                                                                              float *__restrict__ gains) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(FGT) k_filter_one(const double *__restrict__ p
 #pragma unroll
         for (int i = 0; i < BATCH; ++i) {
             const int k = t + FGT * (BATCH * h + i);
-            b[i] = k < NBIN ? psd_bits(__ldg(p + k), k, k_hp) : 0LL;
+            b[i] = k < NBIN ? psd_bits(p[k], k, k_hp) : 0LL;
         }
 #pragma unroll
         for (int i = 0; i < BATCH; ++i)
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(FGT) k_filter_one(const double *__restrict__ p
 #pragma unroll 8
         for (int i = t; i < 1024 + (rho == 0); i += FGT) {
             const int k = 8 * i + rho;
-            const long long b = psd_bits(__ldg(p + k), k, k_hp);
+            const long long b = psd_bits(p[k], k, k_hp);
             dd a = {0.f, 0.f};
             if (b) a = amplitude(b, s);
             amp[row * ARS + i] = make_float2(a.h, a.l);

@@ -60,7 +60,7 @@ constexpr int64_t CL_DIRECT = 16384;
 constexpr int CL_DIRECT_H = 256;
 
 template <bool NAN_STOPS>
-__global__ void __launch_bounds__(CL_T) k_cluster(const float *__restrict__ z, int64_t n_out, int n_int, int h,
+__global__ void __launch_bounds__(CL_T) k_cluster(const float *z, int64_t n_out, int n_int, int h,
                                                   float *__restrict__ stat, uint32_t *__restrict__ flags,
                                                   int *__restrict__ counts, int64_t *__restrict__ idx, int64_t cap,
                                                   int64_t *__restrict__ n_trig) {
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(CL_T) k_cluster(const float *__restrict__ z, i
 
 // grid (tiles): the tile's triggers behind those of the tiles before it.  counts: of every tile, added up here, or
 // (scanned) already an exclusive sum with the total written.
-__global__ void __launch_bounds__(CL_T) k_cluster_write(const uint32_t *__restrict__ flags, const int *__restrict__ counts,
+__global__ void __launch_bounds__(CL_T) k_cluster_write(const uint32_t *flags, const int *counts,
                                                         int scanned, int64_t *__restrict__ idx, int64_t cap,
                                                         int64_t *__restrict__ n_trig) {
     __shared__ int64_t sum[CL_T / 32];

@@ -336,7 +336,7 @@ constexpr int GNS_T = 512;
 constexpr int GNS_U = 3;
 
 template <int GS, bool REG>
-__global__ void __launch_bounds__(GNS_T, 2) k_gn_split(const float *__restrict__ raw, int64_t hs, int hr, int L,
+__global__ void __launch_bounds__(GNS_T, 2) k_gn_split(const float *raw, int64_t hs, int hr, int L,
                                                                  int cp, int lcg, const float *__restrict__ gamma,
                                                                  const float *__restrict__ beta, float eps,
                                                                  const Planes res, int relu, const Planes out) {

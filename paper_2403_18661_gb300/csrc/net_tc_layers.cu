@@ -290,11 +290,11 @@ __device__ __forceinline__ bool issue_stage(int shape, const StageGeo &g) {
 // Residual rows of a channel-major epilogue unit (16 * NQ positions from p_first): lane e of
 // each octet loads rows p_first + 8 b + e + 1 of the octet's chunk (issued one unit ahead).
 template <int NQ>
-__device__ __forceinline__ void ch_res_load(const __nv_bfloat16 *__restrict__ rw8, int p_first, int lane,
+__device__ __forceinline__ void ch_res_load(const __nv_bfloat16 *rw8, int p_first, int lane,
                                             uint4 (&rr)[4]) {
 #pragma unroll
     for (int b = 0; b < 2 * NQ; ++b)
-        rr[b] = __ldg(reinterpret_cast<const uint4 *>(rw8 + (size_t)(p_first + 8 * b + (lane & 7) + 1) * 8));
+        rr[b] = *reinterpret_cast<const uint4 *>(rw8 + (size_t)(p_first + 8 * b + (lane & 7) + 1) * 8);
 }
 
 // Channel-major epilogue of 16 * NQ consecutive positions of the warp's 32 channels: the
@@ -579,14 +579,14 @@ __global__ void __launch_bounds__(LT, 1) k_conv_tc(const LayerArgs a) {
                 const int cg = a.Cout / a.G;
                 const size_t ld = (size_t)(a.Lout + 2) * a.Cout;  // elements per window
                 const size_t cs = (size_t)(a.Lout + 2) * 8;       // elements per chunk
-                const __nv_bfloat16 *__restrict__ rw = a.res ? a.res + (size_t)w * ld : nullptr;
+                const __nv_bfloat16 *rw = a.res ? a.res + (size_t)w * ld : nullptr;
                 // residual units (subtile j, 32 channels from c0) are loaded one unit ahead; the
                 // first is issued before the statistics pass
                 uint4 cur[4], nxt[4];
                 if (rw && hsel < MT) {
                     const size_t o0 = (size_t)(128 * hsel + 32 * q + lane + 1) * 8;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) cur[i] = __ldg(reinterpret_cast<const uint4 *>(rw + o0 + i * cs));
+                    for (int i = 0; i < 4; ++i) cur[i] = *reinterpret_cast<const uint4 *>(rw + o0 + i * cs);
                 }
                 // per-warp group partials: red[e][g] (sum) and red[e][16 + g] (sum of squares)
                 float part;
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(LT, 1) k_conv_tc(const LayerArgs a) {
                                 const size_t on = (size_t)(cn / 8) * cs + (size_t)(128 * jn + 32 * q + lane + 1) * 8;
 #pragma unroll
                                 for (int i = 0; i < 4; ++i)
-                                    nxt[i] = __ldg(reinterpret_cast<const uint4 *>(rw + on + i * cs));
+                                    nxt[i] = *reinterpret_cast<const uint4 *>(rw + on + i * cs);
                             }
                         }
                         uint4 rr[4];
@@ -1242,7 +1242,7 @@ __global__ void __launch_bounds__(STC_T, 2) k_stem_tc(const float *__restrict__ 
 
 // grid (n_win), block 256: logit = fc_b + sum_c fc_w[c] * mean_t x[t][c] (bf16 chunk-major input,
 // C / 8 <= 256 chunks); each thread sums 8 channels of one chunk over a subset of rows
-__global__ void k_head_bf16(const __nv_bfloat16 *__restrict__ x, int L, int C, const float *__restrict__ fc_w,
+__global__ void k_head_bf16(const __nv_bfloat16 *x, int L, int C, const float *__restrict__ fc_w,
                             const float *__restrict__ fc_b, float *__restrict__ logits, int64_t w0) {
     __shared__ float part[256][9];
     const int tid = threadIdx.x, nch = C / 8, tpc = 256 / nch;  // threads per chunk
@@ -1252,7 +1252,7 @@ __global__ void k_head_bf16(const __nv_bfloat16 *__restrict__ x, int L, int C, c
     if (r0 < tpc) {
         const uint4 *xc = reinterpret_cast<const uint4 *>(x + ((int64_t)blockIdx.x * nch + ch) * (L + 2) * 8) + 1;
         for (int r = r0; r < L; r += tpc) {
-            const uint4 u = __ldg(xc + r);
+            const uint4 u = xc[r];
             const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {

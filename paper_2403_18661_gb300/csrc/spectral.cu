@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(PSD_T64) k_psd_mean64(const float *P, int64_t 
 // A thread takes bins k and k + PSD_T as the halves of packed additions (the loads and stores of both coalesce).
 constexpr int PSD_T = 128;
 
-__global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *__restrict__ P, int64_t n_seg, int seg_step, int K,
+__global__ void __launch_bounds__(PSD_T) k_psd_mean(const float *P, int64_t n_seg, int seg_step, int K,
                                                     double *__restrict__ psd, int64_t n_psd) {
     __shared__ float sf[PSD_SEGS];  // 2^(e_s - e_max) of the run's segments
     __shared__ int elo, ehi;
@@ -650,7 +650,7 @@ __device__ __forceinline__ WhitenBlock whiten_block_at(const WhitenLayout &L, in
 // Else the gains come in during the forward transform.
 template <bool EARLY>
 __global__ void __launch_bounds__(r16::NT, 2) k_whiten(const float *__restrict__ x, int64_t n, int64_t x_stride,
-                                                        const float *__restrict__ gains, int64_t n_psd,
+                                                        const float *gains, int64_t n_psd,
                                                         int64_t out_first, int64_t out_len, int64_t epoch_len, int F,
                                                         float *__restrict__ y, int64_t y_stride) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
