@@ -276,10 +276,10 @@ __global__ void k_far_count(const float *sorted, const int64_t *n_dev, int64_t c
     const int64_t n = dev_count(n_dev, cap);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
-    const bool nan = n > 0 && isnan(sorted[0]);
+    const float first = n > 0 ? sorted[0] : 0.f;  // (looked at after the search: its load waits for nothing)
     for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; j < n_fg; j += warps) {
         const float x = fg[j];
-        int64_t lo = nan ? bisect(sorted, n, x) : 0, hi = nan ? lo : n;  // the answer lies in [lo, hi]
+        int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
         while (lo < hi) {
             const int64_t step = (hi - lo + 32) / 33, i = lo + step * (lane + 1) - 1;  // probes, in order
             const uint32_t above = __ballot_sync(0xffffffffu, i < hi && sorted[i] > x);
@@ -288,6 +288,7 @@ __global__ void k_far_count(const float *sorted, const int64_t *n_dev, int64_t c
             lo += step * c;
             hi = c < 32 && nhi < hi ? nhi : hi;
         }
+        if (isnan(first)) lo = bisect(sorted, n, x);
         if (lane == 0) {
             if (n_above) n_above[j] = lo;
             if (far) far[j] = (double)lo / livetime;
