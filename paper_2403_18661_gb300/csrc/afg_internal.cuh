@@ -295,6 +295,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // Error plumbing
 // ----------------------------------------------------------------------------
 int afg_fail(afg_ctx *ctx, int code, const char *fmt, ...);
+cudaError_t allow_smem_of(const void *kernel, size_t bytes);
+template <typename K>
+inline cudaError_t allow_smem(K *kernel, size_t bytes) { return allow_smem_of(reinterpret_cast<const void *>(kernel), bytes); }
 int afg_cuda_fail(afg_ctx *ctx, cudaError_t e, const char *what);
 int afg_ws_reserve(afg_ctx *ctx, int slot, size_t bytes, void **out);
 void afg_ws_release(afg_ctx *ctx, int slot);

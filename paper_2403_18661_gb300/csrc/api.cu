@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "afg_internal.cuh"
 
@@ -26,6 +27,17 @@ int afg_fail(afg_ctx *ctx, int code, const char *fmt, ...) {
 int afg_cuda_fail(afg_ctx *ctx, cudaError_t e, const char *what) {
     return afg_fail(ctx, e == cudaErrorMemoryAllocation ? AFG_ERR_OOM : AFG_ERR_CUDA, "%s: %s (%s)", what,
                     cudaGetErrorString(e), cudaGetErrorName(e));
+}
+
+// Allow a kernel `bytes` of dynamic shared memory on the current device.  The limit belongs to the kernel and the device,
+// not to a context: it is only ever raised, since another context may launch the kernel with more.
+cudaError_t allow_smem_of(const void *kernel, size_t bytes) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // Grow-only workspace slot.  Growing frees the old buffer (synchronising

@@ -494,11 +494,6 @@ void conv_launch(afg_ctx *ctx, const float *in, const float *wt, float *out, int
     KScope ks(ctx, st, KK_CONV_FP32, 2.0 * M * L.cout * K,
               4.0 * ((double)nw * L.lin * L.cin + (double)K * L.cout + (double)M * L.cout));
     constexpr size_t smem = ConvSmem<BM, BN, BK>::bytes;
-    static bool attr_set = false;  // per instantiation; one device per process
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_conv_fp32<BM, BN, TM, TN, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr_set = true;
-    }
     k_conv_fp32<BM, BN, TM, TN, BK><<<grid, 256, smem, st>>>(in, wt, out, M, L.lout, L.lin + 2, L.lout + 2, L.cin,
                                                              L.cout, K, L.stride, off);
 }
@@ -510,6 +505,15 @@ void conv_dispatch(afg_ctx *ctx, const float *in, float *out, int nw, const Conv
     else conv_launch<256, 16, 4, 4, 16>(ctx, in, L.wt, out, nw, L, st);
 }
 
+// Shared-memory limits of the kernels above, at every context's creation
+int fp32_set_attrs(afg_ctx *ctx) {
+    AFG_CUDA(ctx, allow_smem(k_conv_fp32<128, 128, 8, 8, 16>, ConvSmem<128, 128, 16>::bytes));
+    AFG_CUDA(ctx, allow_smem(k_conv_fp32<256, 64, 8, 8, 16>, ConvSmem<256, 64, 16>::bytes));
+    AFG_CUDA(ctx, allow_smem(k_conv_fp32<256, 16, 4, 4, 16>, ConvSmem<256, 16, 16>::bytes));
+    AFG_CUDA(ctx, allow_smem(k_groupnorm_st, GN_ST_MAX4 * 16));
+    return AFG_OK;
+}
+
 // GroupNorm launch with its accounting: one read (+ residual read) and one write of the tile
 void gn_launch(afg_ctx *ctx, float *x, int nw, int L, int C, int G, const float *gamma, const float *beta, float eps,
                const float *res, int relu, float *pool_out, cudaStream_t st) {
@@ -519,11 +523,6 @@ void gn_launch(afg_ctx *ctx, float *x, int nw, int L, int C, int G, const float 
     KScope ks(ctx, st, KK_GROUPNORM, 0.0, bytes);
     const int64_t n4 = (int64_t)L * C / 4;
     if (!pool_out && C % 4 == 0 && C <= 512 && GN_ST % (C / 4) == 0 && n4 >= GN_ST && n4 <= GN_ST_MAX4) {
-        static bool attr_set = false;  // one device per process
-        if (!attr_set) {
-            cudaFuncSetAttribute(k_groupnorm_st, cudaFuncAttributeMaxDynamicSharedMemorySize, GN_ST_MAX4 * 16);
-            attr_set = true;
-        }
         k_groupnorm_st<<<nw, GN_ST, (size_t)n4 * 16, st>>>(x, L, C, G, gamma, beta, eps, res, relu);
     } else {
         k_groupnorm<<<nw, GN_T, 0, st>>>(x, L, C, G, gamma, beta, eps, res, relu, pool_out);
@@ -621,7 +620,7 @@ int net_plan_build(afg_ctx *ctx, const float *weights_host, int64_t n_weights) {
     }
     P.fc_w = d + fc_off;
     P.fc_b = d + fc_off + cin;
-    return AFG_OK;
+    return fp32_set_attrs(ctx);
 }
 
 // Stem conv (reading the windows from the whitened stream) + GroupNorm + ReLU

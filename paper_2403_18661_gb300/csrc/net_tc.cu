@@ -1515,27 +1515,22 @@ int net_tc_prepare(afg_ctx *ctx) {
     AFG_CUDA(ctx, cudaMemcpy(P.tc_wimg, img.data(), ibytes, cudaMemcpyHostToDevice));
     const size_t pbase = pipe_smem(ctx->cfg.win_len, n_conv, k).total;
     const int psmem = (int)(pbase + pipe_seg_cache_cap(pbase) * sizeof(SegDesc));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<8, TP_MT_FIXED, 12, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<8, TP_MT_FIXED, 12, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<8, TP_MT_FIXED, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_pipe<8, TP_MT_FIXED, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<1>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<2>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<4>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<8>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<16>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<8, TP_MT_FIXED, 12, 2>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<8, TP_MT_FIXED, 12, 1>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<8, TP_MT_FIXED, 8, 2>, psmem));
+    AFG_CUDA(ctx, allow_smem(k_tiny_pipe<8, TP_MT_FIXED, 8, 1>, psmem));
     if (ctx->cfg.win_len % (128 * TF_CLUSTER) == 0) {  // list mode on clusters: a quarter window per CTA
         const int smem_c = (int)tiny_smem(ctx->cfg.win_len / TF_CLUSTER, n_conv, k).total + TF_XCH;
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_fused<1, TF_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_c));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_fused<2, TF_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_c));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_fused<4, TF_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_c));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_fused<8, TF_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_c));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_tiny_fused<16, TF_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_c));
+        AFG_CUDA(ctx, allow_smem(k_tiny_fused<1, TF_CLUSTER>, smem_c));
+        AFG_CUDA(ctx, allow_smem(k_tiny_fused<2, TF_CLUSTER>, smem_c));
+        AFG_CUDA(ctx, allow_smem(k_tiny_fused<4, TF_CLUSTER>, smem_c));
+        AFG_CUDA(ctx, allow_smem(k_tiny_fused<8, TF_CLUSTER>, smem_c));
+        AFG_CUDA(ctx, allow_smem(k_tiny_fused<16, TF_CLUSTER>, smem_c));
     }
     return AFG_OK;
 }

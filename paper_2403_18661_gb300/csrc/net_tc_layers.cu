@@ -1508,18 +1508,18 @@ int net_tc_layers_prepare(afg_ctx *ctx) {
         AFG_CUDA(ctx, cudaMemcpy(tp->layers[i].wimg, imgs[i].data(), imgs[i].size() * 2, cudaMemcpyHostToDevice));
         off += (imgs[i].size() * 2 + 1023) / 1024 * 1024;
     }
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_conv_tc<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
+    AFG_CUDA(ctx, allow_smem(k_conv_tc<0, false>, SMEM_LIMIT));
+    AFG_CUDA(ctx, allow_smem(k_conv_tc<0, true>, SMEM_LIMIT));
+    AFG_CUDA(ctx, allow_smem(k_conv_tc<1, false>, SMEM_LIMIT));
+    AFG_CUDA(ctx, allow_smem(k_conv_tc<1, true>, SMEM_LIMIT));
     {
         const ConvLayer &S = P.convs[0];
         const int smem = (int)stem_tc_smem(ctx->cfg.win_len, S.k, S.lout).total;
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_tc<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        AFG_CUDA(ctx, cudaFuncSetAttribute(k_stem_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        AFG_CUDA(ctx, allow_smem(k_stem_tc<2>, smem));
+        AFG_CUDA(ctx, allow_smem(k_stem_tc<4>, smem));
+        AFG_CUDA(ctx, allow_smem(k_stem_tc<8>, smem));
+        AFG_CUDA(ctx, allow_smem(k_stem_tc<16>, smem));
+        AFG_CUDA(ctx, allow_smem(k_stem_tc<32>, smem));
     }
     ctx->tcplan = tp;
     return AFG_OK;

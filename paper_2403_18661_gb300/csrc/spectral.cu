@@ -812,16 +812,12 @@ __global__ void __launch_bounds__(r16::NT_S) k_whiten_multi_s(const WhitenPiece 
                    });
 }
 
-bool g_attrs_set = false;
-
 int set_attrs(afg_ctx *ctx) {
-    if (g_attrs_set) return AFG_OK;
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_periodogram, cudaFuncAttributeMaxDynamicSharedMemorySize, WELCH_SMEM));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM));
-    AFG_CUDA(ctx, cudaFuncSetAttribute(k_whiten_multi_s, cudaFuncAttributeMaxDynamicSharedMemorySize, WHITEN_SMEM_S));
-    g_attrs_set = true;
+    AFG_CUDA(ctx, allow_smem(k_periodogram, WELCH_SMEM));
+    AFG_CUDA(ctx, allow_smem(k_whiten<false>, WHITEN_SMEM));
+    AFG_CUDA(ctx, allow_smem(k_whiten<true>, WHITEN_SMEM));
+    AFG_CUDA(ctx, allow_smem(k_whiten_multi, WHITEN_SMEM));
+    AFG_CUDA(ctx, allow_smem(k_whiten_multi_s, WHITEN_SMEM_S));
     return AFG_OK;
 }
 
@@ -1015,5 +1011,5 @@ cudaError_t launch_psd_on(const float *x, int64_t n, int n_det, int64_t n_psd, i
 cudaError_t prepare_psd_kernels() {
     const cudaError_t e = ensure_tw32();
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_periodogram, cudaFuncAttributeMaxDynamicSharedMemorySize, WELCH_SMEM);
+    return allow_smem(k_periodogram, WELCH_SMEM);
 }
