@@ -48,7 +48,9 @@ extern "C" {
 
 /* precision of the network's convolutions */
 #define AFG_FP32 0 /* FP32 operands and accumulation ("plain"): FP32 FMAs, or, where every width is 64..512 and the
-                      context has no memory budget, exact three-term BF16 products on the tensor cores */
+                      context has no memory budget, each float as three BF16 terms (exact from 2^-110 up, to 2^-134
+                      below) and six of the nine products of two floats on the tensor cores (the other three are below
+                      2^-26 of the product) */
 #define AFG_BF16 1 /* BF16 operands, FP32 accumulation on tcgen05 tensor cores */
 
 typedef struct afg_ctx afg_ctx;

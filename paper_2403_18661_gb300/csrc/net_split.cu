@@ -1,9 +1,10 @@
 // FP32 1D ResNet with GroupNorm on the tensor cores (Sec. II network, widths 64..512): every
-// convolution after the stem is an implicit GEMM of BF16 products whose sum is the FP32 product.
+// convolution after the stem is an implicit GEMM of BF16 products whose sum is the FP32 product to 2^-26 or so.
 //
-// A float is the exact sum of three BF16 values (8 significant bits each: 24 in all), x = x1 + x2 + x3,
-// x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2.  The product of two floats is the nine products
-// x_i w_j, each exact in FP32; the six with i + j <= 4 are formed, the other three are below 2^-26 of
+// A float is the sum of three BF16 values (8 significant bits each: 24 in all), x = x1 + x2 + x3,
+// x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2: exactly for |x| from 2^-110 to the largest float (x1 is
+// held at the largest BF16 number), and to 2^-134, half of BF16's smallest, below.  The product of two floats is the
+// nine products x_i w_j, each exact in FP32; the six with i + j <= 4 are formed, the other three are below 2^-26 of
 // |x w|.  FP32 SIMT FMAs run at 80 TFLOP/s on this GPU, six BF16 products at 1950 / 6 = 325 (k_conv_fp32
 // of net_fp32.cu, at 78 % of the FP32 pipe, and its GroupNorm took 73.4 ms for 1920 ResNet34 windows and
 // 14.2 ms for 333; this path takes 23.9 and 4.44, and its logits are closer to 64-bit ones: relative error
@@ -277,25 +278,10 @@ __global__ void __launch_bounds__(SC_T, 1) k_conv_split(const SplitConvArgs a) {
     }
 }
 
-// Weight image of one convolution from wt [k][cin][cout] (the image is zeroed beforehand).
-__global__ void k_split_weights(const float *__restrict__ wt, int cin, int cout, int k, __nv_bfloat16 *__restrict__ o) {
-    const int n = k * cin * cout;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int co = i % cout, ci = i / cout % cin, r = i / cout / cin;
-        const size_t blk = (size_t)(co / 128) * (cin / SC_KB) + ci / SC_KB;
-        float v = wt[i];
-        for (int p = 0; p < 3; ++p) {
-            const __nv_bfloat16 b = __float2bfloat16_rn(v);
-            v -= __bfloat162float(b);
-            o[((((blk * 3 + p) * 2 + ci % SC_KB / 8) * k + r) * 128 + co % 128) * 8 + ci % 8] = b;
-        }
-    }
-}
-
-// ---------------------------------------------------------------- planes
-// the three BF16 terms of two floats (lo in the low half of each word)
+// the three BF16 terms of two floats (lo in the low half of each word).  The first is at most the largest BF16 number: a
+// float that rounds past it would leave x - inf.
 __device__ __forceinline__ void split3(float lo, float hi, uint32_t &p1, uint32_t &p2, uint32_t &p3) {
-    p1 = tc::pack_bf16x2(lo, hi);
+    p1 = tc::pack_bf16x2_sat(lo, hi);
     lo -= __uint_as_float(p1 << 16);
     hi -= __uint_as_float(p1 & 0xffff0000u);
     p2 = tc::pack_bf16x2(lo, hi);
@@ -303,6 +289,22 @@ __device__ __forceinline__ void split3(float lo, float hi, uint32_t &p1, uint32_
     hi -= __uint_as_float(p2 & 0xffff0000u);
     p3 = tc::pack_bf16x2(lo, hi);
 }
+
+// Weight image of one convolution from wt [k][cin][cout] (the image is zeroed beforehand).
+__global__ void k_split_weights(const float *__restrict__ wt, int cin, int cout, int k, __nv_bfloat16 *__restrict__ o) {
+    const int n = k * cin * cout;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int co = i % cout, ci = i / cout % cin, r = i / cout / cin;
+        const size_t blk = (size_t)(co / 128) * (cin / SC_KB) + ci / SC_KB;
+        uint32_t b[3];
+        split3(wt[i], 0.f, b[0], b[1], b[2]);
+        for (int p = 0; p < 3; ++p)
+            o[((((blk * 3 + p) * 2 + ci % SC_KB / 8) * k + r) * 128 + co % 128) * 8 + ci % 8] =
+                __ushort_as_bfloat16((unsigned short)b[p]);
+    }
+}
+
+// ---------------------------------------------------------------- planes
 __device__ __forceinline__ float2 join3(uint32_t p1, uint32_t p2, uint32_t p3) {  // exact: the sum is the float
     return make_float2((__uint_as_float(p1 << 16) + __uint_as_float(p2 << 16)) + __uint_as_float(p3 << 16),
                        (__uint_as_float(p1 & 0xffff0000u) + __uint_as_float(p2 & 0xffff0000u)) +

@@ -123,3 +123,31 @@ def test_split_on_a_device_with_little_room():
         del filler
         torch.cuda.empty_cache()
     ctx.close()
+
+
+def test_split_of_floats_that_round_past_the_bf16_range():
+    """Finite floats above the largest BF16 number, as activations (a stem bias of 3.4e38, read by convolutions with
+    weights of 2^-126) and as weights (times a channel that is zero): finite in FP32, so finite here."""
+    net = inputs.NetSpec(stem_k=3, stem_stride=2, stem_pool=0, widths=(64, 64), blocks=(1, 1), groups=32)
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=256)
+    big = np.float32(3.4e38)
+    w = inputs.make_weights(net, 5)
+    parts = np.split(w, np.cumsum([int(np.prod(s)) for _, s in inputs.weight_shapes(net)])[:-1])
+    parts = [p.reshape(s).copy() for p, (_, s) in zip(parts, inputs.weight_shapes(net))]
+    stem_w, gamma, beta, c1 = parts[:4]
+    gamma[:4], beta[0], beta[1], beta[2:4] = 0.0, big, -1.0, 1.0
+    convs = [p for p in parts if p.ndim == 3 and p.shape[1] == 64]
+    for p in (convs[0], convs[2], convs[4]):  # what reads the stem's output, or its residual
+        p[:, 0] = np.sign(p[:, 0]) * np.float32(2.0 ** -126)
+    c1[:, 1] = np.where(np.arange(3) % 2, big, -big)
+    w = np.concatenate([p.ravel() for p in parts]).astype(np.float32)
+    y = np.random.default_rng(2).standard_normal((2, 400)).astype(np.float32)
+    ctx = abi.Context(wl, w)
+    ctx.profile_enable()
+    z = ctx.infer_windows(torch.from_numpy(y).cuda(), 0, 48, 3).cpu().numpy()
+    assert any(k["name"] == "conv_gemm_fp32_split_tcgen05" for k in ctx.profile_read())
+    ctx.sync()
+    for j in range(3):
+        want = orc.network(net, w, y[:, 48 * j:48 * j + 256].astype(np.float64))
+        assert np.isfinite(want) and abs(z[j] - want) <= LOGIT_TOL * (1 + abs(want)), (j, z[j], want)
+    ctx.close()
