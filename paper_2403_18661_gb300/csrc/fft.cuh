@@ -15,10 +15,6 @@
 
 #include "afg_internal.cuh"
 
-template <typename T> struct Cx;
-template <> struct Cx<float> { using t = float2; };
-template <> struct Cx<double> { using t = double2; };
-
 template <typename C> __device__ __forceinline__ C cmk(decltype(C::x) a, decltype(C::x) b) { C r; r.x = a; r.y = b; return r; }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return cmk<C>(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return cmk<C>(a.x - b.x, a.y - b.y); }
@@ -69,10 +65,10 @@ template <typename C, int SIGN> __device__ __forceinline__ void dft8(C *v) {
     v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
 }
 
-// One Stockham pass of radix R over LEN points held in shared memory `d`.
-template <typename C, int R, int SIGN, int NT, int LEN = NC>
+// One Stockham pass of radix R (8 or 2) over the NC points held in shared memory `d`.
+template <typename C, int R, int SIGN, int NT>
 __device__ __forceinline__ void stockham_pass(C *d, int Ns, const C *tw) {
-    constexpr int NB = LEN / R;         // butterflies in the pass
+    constexpr int NB = NC / R;          // butterflies in the pass
     constexpr int BPT = (NB + NT - 1) / NT;
     C v[BPT][R];
     const int tid = threadIdx.x;
@@ -90,7 +86,6 @@ __device__ __forceinline__ void stockham_pass(C *d, int Ns, const C *tw) {
                 for (int r = 1; r < R; ++r) v[q][r] = cmul(v[q][r], twiddle<C, SIGN>(tw, r * k * tscale));
             }
             if (R == 8) dft8<C, SIGN>(v[q]);
-            else if (R == 4) dft4<C, SIGN>(v[q][0], v[q][1], v[q][2], v[q][3]);
             else dft2<C, SIGN>(v[q][0], v[q][1]);
         }
     }
