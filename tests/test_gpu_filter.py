@@ -56,3 +56,29 @@ def test_filters_match_float64_taps(n_det, n_psd, fir, f_hp, scale, holes):
             want[EPOCH // 2 - half:EPOCH // 2 + half] = float(amp) * _taps(clean[d, e], wl.fs, f_hp, fir)
             assert np.linalg.norm(y[d, e] - want) <= RTOL * np.linalg.norm(want), (d, e)
     ctx.close()
+
+
+# filters longer than the float-pair build's, few enough that the whitening's forward transforms run beside it, and more
+@pytest.mark.parametrize("n_det,n_psd,fir", [(1, 1, 2050), (2, 1, 4096), (2, 3, 4096), (1, 2, 8192), (1, 153, 4096)])
+def test_long_filters_behind_the_early_whitening(n_det, n_psd, fir):
+    """Strain written by the kernel just before the call; the impulse of each epoch returns its taps, call after call."""
+    wl = dataclasses.replace(inputs.PLAIN_64S, fir_len=fir, f_highpass=32.0)
+    rng = np.random.default_rng(fir + n_psd)
+    shape = inputs.NoiseModel().psd(np.arange(NBIN) * wl.fs / NFFT) / 1e-46
+    psd = 1e-46 * shape * rng.gamma(15.0, 1 / 15.0, (n_det, n_psd, NBIN))
+    half, out_len = fir // 2, n_psd * EPOCH
+    x = torch.zeros((n_det, out_len + 2 * half), dtype=torch.float32, device="cuda")
+    at = torch.arange(n_psd, device="cuda") * EPOCH + half + EPOCH // 2
+    psd_d = torch.from_numpy(psd).cuda()
+    ctx = abi.Context(wl, inputs.make_weights(wl.net, 1))
+    for amp in (1e-23, 2e-23, 3e-23):
+        amp = np.float32(amp)
+        x[:, at] = float(amp)
+        y = ctx.whiten(x, psd_d, half, out_len, epoch_len=EPOCH)
+        y = y.cpu().numpy().astype(np.float64).reshape(n_det, n_psd, EPOCH)
+        for d in range(n_det):
+            for e in sorted({0, 1, n_psd // 2, n_psd - 1} & set(range(n_psd))):
+                want = np.zeros(EPOCH)
+                want[EPOCH // 2 - half:EPOCH // 2 + half] = float(amp) * _taps(psd[d, e], wl.fs, 32.0, fir)
+                assert np.linalg.norm(y[d, e] - want) <= RTOL * np.linalg.norm(want), (d, e)
+    ctx.close()
