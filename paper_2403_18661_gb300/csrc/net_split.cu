@@ -858,24 +858,23 @@ static int split_reserve(afg_ctx *ctx, int64_t nw, __nv_bfloat16 *(&act)[4], flo
     return rc;
 }
 
-// The workspaces of windows() windows.  Where the device has no room for them the sequences become shorter, for good.
-template <typename F>
-static int split_fit(afg_ctx *ctx, F windows, __nv_bfloat16 *(&act)[4], float *&raw) {
+// The workspaces of a call of n_win windows, and so of any shorter one.  (Not those of its sequence: 1025 windows go in
+// sequences of 513, but 1024 in one, and a call inside a caller's capture may not grow what a longer one left.)  Where
+// the device has no room for them the sequences become shorter, for good.
+static int split_fit(afg_ctx *ctx, int64_t n_win, __nv_bfloat16 *(&act)[4], float *&raw) {
     int64_t &most = ctx->splitplan->max_chunk;
     int rc;
-    while ((rc = split_reserve(ctx, windows(), act, raw)) == AFG_ERR_OOM && most > 1) {
-        most = std::max<int64_t>(1, std::min(most, windows()) / 2);
+    while ((rc = split_reserve(ctx, std::min(n_win, most), act, raw)) == AFG_ERR_OOM && most > 1) {
+        most = std::max<int64_t>(1, std::min(most, n_win) / 2);
         for (int slot : {(int)WS_ACT0, (int)WS_ACT1, (int)WS_ACT2, (int)WS_ACT3, (int)WS_RAW}) afg_ws_release(ctx, slot);
     }
     return rc;
 }
 
-// What any call of up to n_win windows uses.  (Not the sequence of n_win itself: 1025 windows go in sequences of 513,
-// but 1024 in one.)
 int net_split_reserve(afg_ctx *ctx, int64_t n_win) {
     __nv_bfloat16 *act[4];
     float *raw;
-    return split_fit(ctx, [&] { return std::min<int64_t>(std::max<int64_t>(1, n_win), ctx->splitplan->max_chunk); }, act, raw);
+    return split_fit(ctx, std::max<int64_t>(1, n_win), act, raw);
 }
 
 static cudaError_t split_conv(afg_ctx *ctx, int i, const Planes &in, float *raw, int64_t nw, cudaStream_t st) {
@@ -940,7 +939,7 @@ int launch_infer_split(afg_ctx *ctx, const float *y, int64_t n_y, int64_t y_stri
     const int W = ctx->cfg.win_len;
     __nv_bfloat16 *act[4];
     float *raw;
-    int rc = split_fit(ctx, [&] { return split_chunk(ctx, n_win); }, act, raw);
+    int rc = split_fit(ctx, n_win, act, raw);
     if (rc) return rc;
     const int64_t chunk = split_chunk(ctx, n_win);
     const Planes none = {nullptr, 0, 0, 0, 0};

@@ -151,3 +151,35 @@ def test_split_of_floats_that_round_past_the_bf16_range():
         want = orc.network(net, w, y[:, 48 * j:48 * j + 256].astype(np.float64))
         assert np.isfinite(want) and abs(z[j] - want) <= LOGIT_TOL * (1 + abs(want)), (j, z[j], want)
     ctx.close()
+
+
+def test_split_workspaces_of_a_call_serve_shorter_ones():
+    """1025 windows go in two sequences of 513, 1000 in one of 1000: the second call, here inside a capture, finds its
+    workspaces reserved by the first."""
+    net = inputs.NetSpec(stem_k=3, stem_stride=2, stem_pool=1, widths=(64,), blocks=(1,), groups=16)
+    wl = dataclasses.replace(inputs.PLAIN_64S, net=net, win_len=256)
+    w = inputs.make_weights(net, 3)
+    y = torch.randn((2, 1024 * 16 + 256), device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    other = abi.Context(wl, w)
+    want = other.infer_windows(y, 0, 16, 1000)
+    ctx = abi.Context(wl, w)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        ctx.infer_windows(y, 0, 16, 1025, stream=s)
+        out = torch.zeros(1000, device="cuda")
+        s.synchronize()
+        held = ctx.bytes_held
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            ctx.infer_windows(y, 0, 16, 1000, out=out, stream=s)
+        assert ctx.bytes_held == held
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            s.synchronize()
+            assert torch.equal(out, want)
+    del graph
+    for c in (ctx, other):
+        c.sync()
+        c.close()
